@@ -235,8 +235,9 @@ size_t loglike_layout(const FftPlan& p, const OptsN& o, int w, int wave, Carve* 
   LoglikeBufs t;
   t.wc = cv.take<WalkerC>(w);
   t.knots = cv.take<Knot>((size_t)w * (nk + 1));
+  t.orb = cv.take<char>((size_t)w * orbit_bytes(p.n, o.ks));
   t.ivs = cv.take<char>(o.precision ? (size_t)w * nk * kIvMBytes : 0);
-  t.lisa = cv.take<double>((size_t)(p.n / 256) * 8);
+  t.lisa = cv.take<double>(lisa_len(p.n, o.ks));
   t.dtab = cv.take<char>((size_t)w * p.n1 * cs);
   t.rtab = cv.take<char>((size_t)w * p.n2 * cs);
   t.partial = cv.take<double2>((size_t)w * p.n2);
@@ -327,12 +328,15 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
     launch_wave(b.knots + (size_t)j0 * (nk + 1), b.wc + j0, gw, p.n, ds->dt, ds->t0, o, zg, false, ctx->bt,
                 b.lisa, b.ivs + (size_t)j0 * nk * kIvMBytes, st);
   };
+  const size_t ob = orbit_bytes(p.n, o.ks);
   auto orbit_of = [&](int j0, int gw, cudaStream_t st) {
     Knot* kj = b.knots + (size_t)j0 * (nk + 1);
-    { KTimer t(pf, EMRI_K_ORBIT, st); launch_orbit(b.wc + j0, gw, p.n, ds->dt, ds->t0, o, kj, ctx->mcpi, st); }
+    KTimer t(pf, EMRI_K_ORBIT, st);
+    nl += launch_orbit(b.wc + j0, gw, p.n, ds->dt, lisa_knots(b.lisa, p.n), o, kj, ctx->mcpi, b.orb + (size_t)j0 * ob,
+                       st);
     if (f32) {
-      KTimer t(pf, EMRI_K_ORBIT, st);
       launch_intervals_mixed(kj, gw, p.n, o.ks, ds->dt, b.ivs + (size_t)j0 * nk * kIvMBytes, st);
+      ++nl;
     }
   };
   if (pipe == 0) {
@@ -346,9 +350,9 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   { KTimer t(pf, EMRI_K_PROLOGUE, s); launch_prologue(theta, ld, w, p.n, ds->dt, o, ctx->gl, b.wc, s); }
   { KTimer t(pf, EMRI_K_DELAY, s); launch_delay_table(b.wc, w, p.n1, p.n2, f32, b.dtab, b.rtab, s); }
   if (pipe <= 1) {
+    launch_lisa(p.n, o.ks, ds->t0, ds->dt, b.lisa, s);
     orbit_of(0, w, s);
-    launch_lisa_tiles(p.n, ds->t0, ds->dt, b.lisa, s);
-    nl += f32 ? 6 : 5;
+    nl += 4;
     for (int i0 = 0; i0 < w; i0 += wave) {
       const int ww = std::min(wave, w - i0);
       wave_of(i0, ww, b.z, s);
@@ -358,7 +362,7 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   } else {
     int rc = pipe_resources(ctx);
     if (rc) return rc;
-    launch_lisa_tiles(p.n, ds->t0, ds->dt, b.lisa, s);
+    launch_lisa(p.n, o.ks, ds->t0, ds->dt, b.lisa, s);
     nl += 4;
     cudaStream_t so = ctx->pstream[0], sf = ctx->pstream[1];
     cudaEvent_t* ev = ctx->pev.data();
@@ -376,8 +380,6 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
     cudaEventRecord(ev[1], so);
     if (g0 < w) orbit_of(g0, w - g0, so);
     cudaEventRecord(ev[3], so);
-    nl += f32 ? 2 : 1;
-    if (g0 < w) nl += f32 ? 2 : 1;
     int prev_gs = 0, prev_g = 0;   // group size and count of the previous wave
     for (int i0 = 0, wv = 0; i0 < w; i0 += wave, ++wv) {
       const int ww = std::min(wave, w - i0);
@@ -798,25 +800,31 @@ extern "C" int emri_ak_waveform(emri_ctx* ctx, const emri_grid* grid, const doub
   Carve probe(nullptr);
   probe.take<WalkerC>(w);
   probe.take<Knot>((size_t)w * (nk + 1));
+  probe.take<char>((size_t)w * orbit_bytes(grid->n, o.ks));
   probe.take<char>(o.precision ? (size_t)w * nk * kIvMBytes : 0);
-  probe.take<double>((size_t)(grid->n / 256) * 8);
+  probe.take<double>(lisa_len(grid->n, o.ks));
   if ((rc = ctx->ws.reserve(ctx, probe.off + 512, s))) return rc;
   ctx->ws.acquire(s);
   Carve cv(ctx->ws.ptr);
   WalkerC* wc = cv.take<WalkerC>(w);
   Knot* kn = cv.take<Knot>((size_t)w * (nk + 1));
+  char* orb = cv.take<char>((size_t)w * orbit_bytes(grid->n, o.ks));
   char* ivs = cv.take<char>(o.precision ? (size_t)w * nk * kIvMBytes : 0);
-  double* lisa = cv.take<double>((size_t)(grid->n / 256) * 8);
+  double* lisa = cv.take<double>(lisa_len(grid->n, o.ks));
   Profiler* pf = &ctx->prof;
   { KTimer t(pf, EMRI_K_PROLOGUE, s); launch_prologue(theta, w, w, grid->n, grid->dt, o, ctx->gl, wc, s); }
-  { KTimer t(pf, EMRI_K_ORBIT, s); launch_orbit(wc, w, grid->n, grid->dt, grid->t0, o, kn, ctx->mcpi, s); }
-  launch_lisa_tiles(grid->n, grid->t0, grid->dt, lisa, s);
+  launch_lisa(grid->n, o.ks, grid->t0, grid->dt, lisa, s);
+  int64_t nl = 0;
+  {
+    KTimer t(pf, EMRI_K_ORBIT, s);
+    nl = launch_orbit(wc, w, grid->n, grid->dt, lisa_knots(lisa, grid->n), o, kn, ctx->mcpi, orb, s);
+  }
   if (o.precision) launch_intervals_mixed(kn, w, grid->n, o.ks, grid->dt, ivs, s);
   { KTimer t(pf, EMRI_K_WAVE, s); launch_wave(kn, wc, w, grid->n, grid->dt, grid->t0, o, z_out, true, ctx->bt, lisa, ivs, s); }
   if (status) cudaMemcpy2DAsync(status, sizeof(uint32_t), &wc[0].status, sizeof(WalkerC), sizeof(uint32_t), w,
                                 cudaMemcpyDeviceToDevice, s);
   ctx->ws.release(s);
-  ctx->launches += o.precision ? 5 : 4;
+  ctx->launches += nl + (o.precision ? 4 : 3);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "waveform launch");
   return EMRI_OK;

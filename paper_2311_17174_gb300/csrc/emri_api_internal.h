@@ -54,8 +54,9 @@ struct Carve {
 struct LoglikeBufs {
   WalkerC* wc;
   Knot* knots;
+  char* orb;       // orbit solver state [w][orbit_bytes]
   char* ivs;       // mixed interval records [w][n/ks]
-  double* lisa;    // per-tile LISA-phase table [n/256][8]
+  double* lisa;    // LISA-phase table (lisa_len)
   char* dtab;
   char* rtab;      // per-walker row delay factors [w][n2]
   double2* partial;

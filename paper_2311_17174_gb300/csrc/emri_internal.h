@@ -71,18 +71,25 @@ void launch_fdprop(const double* theta, int64_t ld, int w, int64_t n, double dt,
                    double fstar, const double* coef, int64_t ldc, FdW* fd, cudaStream_t s);
 
 // orbit: knots[w][nk+1], nk = n / ks
-// mcpi_tab: Chebyshev-Picard tables (qn then qk), required
-void launch_orbit(WalkerC* wc, int w, int64_t n, double dt, double t0, const OptsN& o, Knot* knots,
-                  const double* mcpi_tab, cudaStream_t s);
+// mcpi_tab: Chebyshev-Picard tables (qn then qk), required; orb: solver state
+// of the walkers, orbit_bytes(n, ks) each; cs: cos, sin of the LISA orbital
+// phase at the knots (lisa_knots).  Returns the number of launches.
+int launch_orbit(WalkerC* wc, int w, int64_t n, double dt, const double2* cs, const OptsN& o, Knot* knots,
+                 const double* mcpi_tab, char* orb, cudaStream_t s);
+size_t orbit_bytes(int64_t n, int ks);
 
 // waveform: z[w][n] (double2 or float2); unit_scale multiplies by mu_s c (cm units)
-// lisa: per-tile phibar table [n/256][8] (launch_lisa_tiles); ivs: mixed
+// lisa: LISA orbital phase table (launch_lisa); ivs: mixed
 // interval records [w][n/ks] (launch_intervals_mixed; unused for FP64)
 void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double dt, double t0,
                  const OptsN& o, void* z, bool unit_scale, const BesselTab& bt, const double* lisa, const void* ivs,
                  cudaStream_t s);
 void launch_intervals_mixed(const Knot* knots, int w, int64_t n, int ks, double dt, void* ivs, cudaStream_t s);
-void launch_lisa_tiles(int64_t n, double t0, double dt, double* tab, cudaStream_t s);
+// cos, sin of the LISA orbital phase at the pattern-fit nodes of each
+// 256-sample tile, [n/256][8], then at the knots, [n/ks + 1][2]
+inline size_t lisa_len(int64_t n, int ks) { return (size_t)(n / 256) * 8 + (size_t)(n / ks + 1) * 2; }
+inline const double2* lisa_knots(const double* tab, int64_t n) { return (const double2*)(tab + (n / 256) * 8); }
+void launch_lisa(int64_t n, int ks, double t0, double dt, double* tab, cudaStream_t s);
 constexpr size_t kIvMBytes = 104;
 
 // FFT pass 1 (columns, in place, with the inter-pass twiddle); sign -1 forward, +1 inverse
