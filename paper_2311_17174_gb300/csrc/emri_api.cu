@@ -352,7 +352,7 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   if (pipe <= 1) {
     launch_lisa(p.n, o.ks, ds->t0, ds->dt, b.lisa, s);
     orbit_of(0, w, s);
-    nl += 4;
+    nl += 3;
     for (int i0 = 0; i0 < w; i0 += wave) {
       const int ww = std::min(wave, w - i0);
       wave_of(i0, ww, b.z, s);
@@ -363,7 +363,7 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
     int rc = pipe_resources(ctx);
     if (rc) return rc;
     launch_lisa(p.n, o.ks, ds->t0, ds->dt, b.lisa, s);
-    nl += 4;
+    nl += 3;
     cudaStream_t so = ctx->pstream[0], sf = ctx->pstream[1];
     cudaEvent_t* ev = ctx->pev.data();
     cudaEventRecord(ev[0], s);

@@ -2,6 +2,7 @@
 // double-double arithmetic shared by the libemri kernels.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace emri {
@@ -131,13 +132,13 @@ __host__ __device__ __forceinline__ dd quick_two_sum(double a, double b) {
   return dd{s, e};
 }
 
-__device__ __forceinline__ dd two_prod(double a, double b) {
+__host__ __device__ __forceinline__ dd two_prod(double a, double b) {
   double p = a * b;
   double e = fma(a, b, -p);
   return dd{p, e};
 }
 
-__device__ __forceinline__ dd dd_add(dd a, dd b) {
+__host__ __device__ __forceinline__ dd dd_add(dd a, dd b) {
   dd s = two_sum(a.hi, b.hi);
   dd t = two_sum(a.lo, b.lo);
   s.lo += t.hi;
@@ -146,38 +147,42 @@ __device__ __forceinline__ dd dd_add(dd a, dd b) {
   return quick_two_sum(s.hi, s.lo);
 }
 
-__device__ __forceinline__ dd dd_neg(dd a) { return dd{-a.hi, -a.lo}; }
-__device__ __forceinline__ dd dd_sub(dd a, dd b) { return dd_add(a, dd_neg(b)); }
+__host__ __device__ __forceinline__ dd dd_neg(dd a) { return dd{-a.hi, -a.lo}; }
+__host__ __device__ __forceinline__ dd dd_sub(dd a, dd b) { return dd_add(a, dd_neg(b)); }
 
-__device__ __forceinline__ dd dd_add_d(dd a, double b) {
+__host__ __device__ __forceinline__ dd dd_add_d(dd a, double b) {
   dd s = two_sum(a.hi, b);
   s.lo += a.lo;
   return quick_two_sum(s.hi, s.lo);
 }
 
-__device__ __forceinline__ dd dd_mul(dd a, dd b) {
+__host__ __device__ __forceinline__ dd dd_mul(dd a, dd b) {
   dd p = two_prod(a.hi, b.hi);
   p.lo += a.hi * b.lo + a.lo * b.hi;
   return quick_two_sum(p.hi, p.lo);
 }
 
-__device__ __forceinline__ dd dd_mul_d(dd a, double b) {
+__host__ __device__ __forceinline__ dd dd_mul_d(dd a, double b) {
   dd p = two_prod(a.hi, b);
   p.lo += a.lo * b;
   return quick_two_sum(p.hi, p.lo);
 }
 
-__device__ __forceinline__ dd dd_div(dd a, dd b) {
-  double q1 = a.hi / b.hi;
+// three quotient digits with one reciprocal (a double division is ~15 FP64
+// instructions on the device); each digit is off by a few ulps at most and
+// the next one takes up the remainder
+__host__ __device__ __forceinline__ dd dd_div(dd a, dd b) {
+  const double inv = 1.0 / b.hi;
+  double q1 = a.hi * inv;
   dd r = dd_sub(a, dd_mul_d(b, q1));
-  double q2 = r.hi / b.hi;
+  double q2 = r.hi * inv;
   r = dd_sub(r, dd_mul_d(b, q2));
-  double q3 = r.hi / b.hi;
+  double q3 = r.hi * inv;
   dd q = quick_two_sum(q1, q2);
   return dd_add_d(q, q3);
 }
 
-__device__ __forceinline__ dd dd_sqrt(dd a) {
+__host__ __device__ __forceinline__ dd dd_sqrt(dd a) {
   // one Newton step from the double square root: s + (a - s^2) / (2 s)
   if (a.hi <= 0.0) return dd{0.0, 0.0};
   double s = sqrt(a.hi);
@@ -185,27 +190,30 @@ __device__ __forceinline__ dd dd_sqrt(dd a) {
   return dd_add_d(dd{s, 0.0}, r.hi / (2.0 * s));
 }
 
-// exp of a dd argument: x = k ln2 + r, r reduced by 2^-9, Taylor series to
-// order 14 in dd, then 9 squarings and the 2^k scale.
-__device__ inline dd dd_exp(dd x) {
+// exp of a dd argument: x = k ln2 + r, r reduced by 2^-9 (|r| < 6.8e-4),
+// exp(r) - 1 by its Taylor series -- in dd up to r^4, the rest, below 1e-15 of
+// the sum, in double -- then 9 squarings and the 2^k scale.  Relative error
+// ~1e-31.
+__host__ __device__ inline dd dd_exp(dd x) {
   const dd ln2{0.6931471805599453, 2.3190468138462996e-17};
-  double k = rint(x.hi / ln2.hi);
+  const double k = rint(x.hi / ln2.hi);
   dd r = dd_sub(x, dd_mul_d(ln2, k));
-  r = dd{ldexp(r.hi, -9), ldexp(r.lo, -9)};
-  dd term = r, sum = r;
-  for (int i = 2; i <= 14; ++i) {
-    term = dd_div(dd_mul(term, r), dd_make((double)i));
-    sum = dd_add(sum, term);
-  }
+  r = dd{r.hi * 0x1p-9, r.lo * 0x1p-9};
+  const double t = fma(r.hi, fma(r.hi, fma(r.hi, 1.0 / 40320.0, 1.0 / 5040.0), 1.0 / 720.0), 1.0 / 120.0);
+  dd p = dd_add(dd{0.041666666666666664, 2.3129646346357427e-18}, dd_mul_d(r, t));
+  p = dd_add(dd{0.16666666666666666, 9.25185853854297e-18}, dd_mul(r, p));
+  p = dd_add_d(dd_mul(r, p), 0.5);
+  p = dd_add_d(dd_mul(r, p), 1.0);
+  dd sum = dd_mul(r, p);
   // exp(r) - 1 = sum; square 9 times: (1 + s)^2 - 1 = 2 s + s^2
-  for (int i = 0; i < 9; ++i) sum = dd_add(dd_mul_d(sum, 2.0), dd_mul(sum, sum));
+  for (int i = 0; i < 9; ++i) sum = dd_add(dd{2.0 * sum.hi, 2.0 * sum.lo}, dd_mul(sum, sum));
   dd e = dd_add_d(sum, 1.0);
   return dd{ldexp(e.hi, (int)k), ldexp(e.lo, (int)k)};
 }
 
 // log of a positive dd: y0 = log(hi), then one Newton step y0 + (a e^-y0 - 1)
 // with the second-order term, accurate to dd precision.
-__device__ inline dd dd_log(dd a) {
+__host__ __device__ inline dd dd_log(dd a) {
   double y0 = log(a.hi);
   dd t = dd_mul(a, dd_exp(dd{-y0, 0.0}));   // ~ 1 + eps
   dd u = dd_add_d(t, -1.0);
@@ -214,13 +222,13 @@ __device__ inline dd dd_log(dd a) {
 }
 
 // asinh(a) = log(a + sqrt(a^2 + 1)) for a >= 0
-__device__ inline dd dd_asinh(dd a) {
+__host__ __device__ inline dd dd_asinh(dd a) {
   dd s = dd_sqrt(dd_add_d(dd_mul(a, a), 1.0));
   return dd_log(dd_add(a, s));
 }
 
 // fractional part in [0, 1) of a dd value
-__device__ inline dd dd_frac(dd a) {
+__host__ __device__ inline dd dd_frac(dd a) {
   double f = floor(a.hi);
   dd r = dd_add_d(dd{a.hi - f, 0.0}, a.lo);   // a.hi - f is exact
   if (r.hi < 0.0) r = dd_add_d(r, 1.0);
