@@ -31,6 +31,7 @@
 // no FP64 instruction runs per sample; the rest is FP32.
 #include <vector>
 #include "emri_common.cuh"
+#include "fx64.cuh"
 #include "emri_internal.h"
 
 namespace emri {
@@ -122,6 +123,8 @@ int upload_bessel_tables(const BesselTab& t) {
 // cycles; filled from the host (long double) at context creation.
 constexpr int kExpLen = 512;
 __device__ double2 g_exp512[kExpLen];
+// exp(2 pi i k / 1024) in Q62 for the fixed-point sin/cos
+__device__ fx::Trig g_trig[fx::kTrigLen];
 
 int upload_exp512() {
   double2 h[kExpLen];
@@ -130,7 +133,15 @@ int upload_exp512() {
     const long double a = 2.0L * pi * (long double)k / (long double)kExpLen;
     h[k] = make_double2((double)cosl(a), (double)sinl(a));
   }
-  return cudaMemcpyToSymbol(g_exp512, h, sizeof(h)) == cudaSuccess ? 0 : -1;
+  std::vector<fx::Trig> q(fx::kTrigLen);
+  for (int k = 0; k < fx::kTrigLen; ++k) {
+    const long double a = 2.0L * pi * (long double)k / (long double)fx::kTrigLen;
+    q[k].c = llrintl(cosl(a) * 0x1p62L);
+    q[k].s = llrintl(sinl(a) * 0x1p62L);
+  }
+  const bool ok = cudaMemcpyToSymbol(g_exp512, h, sizeof(h)) == cudaSuccess &&
+                  cudaMemcpyToSymbol(g_trig, q.data(), q.size() * sizeof(fx::Trig)) == cudaSuccess;
+  return ok ? 0 : -1;
 }
 
 // cos(2 pi f), sin(2 pi f) for a phase f in cycles (|f| < 2^20; whole cycles
@@ -637,46 +648,15 @@ constexpr double kPatternFitDtMaxM = 1024.0;    // [s]; fit error < 1e-7 below
 // kernel's at one fit per tile, drops four-fold.
 constexpr int kSegF = 1024;
 
-__global__ void __launch_bounds__(kTile, 2) k2_wave_f64(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
-                                                        int64_t n, double dt, double t0, int ks, int n_max,
-                                                        double2* __restrict__ z, int unit_scale, int exact_f,
-                                                        const double* __restrict__ bc, const double* __restrict__ ifact,
-                                                        const double* __restrict__ lisa) {
+// The samples of a segment in double, for the segments the fixed-point form
+// does not take (wave_fixed_ok): long sample intervals, whose antenna patterns
+// are exact per sample, and orbits or geometries outside its ranges.
+__device__ __noinline__ void wave_samples_f64(const IvD* iv, const double* bq, const double (*fq)[4][4],
+                                              const Geo<double>& g, int64_t j0, int64_t kfirst, int64_t jplunge,
+                                              int span, double dt, double t0, int ks, int n_max, double scale,
+                                              int exact_f, double2* __restrict__ z) {
   constexpr int kTiles = kSegF / kTile;
-  __shared__ IvD iv[kSegF / 64];
-  __shared__ double bnode[3 * 32 * 3];
-  __shared__ double bq[32 * 9];
-  __shared__ double fn[kTiles][4][4];   // the four patterns at the four fit nodes of each tile
-  __shared__ double fq[kTiles][4][4];   // their cubics in (t mod 256) / 256
-  __shared__ double2 ex[kExpLen];
-  __shared__ Geo<double> g;
-  const int wk = blockIdx.y;
-  const WalkerC& C = wcs[wk];
-  const int64_t nk = n / ks;
-  const Knot* kn = knots + (int64_t)wk * (nk + 1);
-  const int64_t j0 = (int64_t)blockIdx.x * kSegF;
-  const int64_t kfirst = j0 / ks;
-  const int ni = ks >= kSegF ? 1 : kSegF / ks;
   const int t = threadIdx.x;
-  const double h = (double)ks * dt;
-  const double scale = unit_scale ? C.gd.amp_scale : 1.0;
-  if (t < ni) build_iv(kn[kfirst + t], kn[kfirst + t + 1], h, iv[t]);
-  if (t >= 224 && t < 224 + 4 * kTiles && !exact_f) {   // node q of tile tt
-    const int i = t - 224, tt = i / 4, q = i % 4;
-    const double* L = lisa + ((int64_t)blockIdx.x * kTiles + tt) * 8 + 2 * q;
-    antenna_fixed<double>(C.gd, L[0], L[1], scale, fn[tt][q]);
-  }
-  if (t == 160) g = C.gd;
-  for (int i = t; i < kExpLen; i += kTile) ex[i] = g_exp512[i];
-  __syncthreads();
-  if (t >= 224 && t < 224 + 4 * kTiles && !exact_f) {   // pattern q of tile tt
-    const int i = t - 224, tt = i / 4, q = i % 4;
-    fit_cubic4<double>(fn[tt][0][q], fn[tt][1][q], fn[tt][2][q], fn[tt][3][q], fq[tt][q]);
-  }
-  const int64_t jplunge = C.j_plunge;
-  const int span = tile_span(j0, jplunge, kSegF);
-  tile_harmonics<double, IvD>(iv, ni, j0, kfirst, ks, n_max, span, bnode, bq, bc, ifact);
-  __syncthreads();
   const double inv_span = 1.0 / (double)span;
   const int lks = __ffs(ks) - 1;   // ks: a power of two
   const double so = (double)t * (1.0 / kTile);
@@ -707,14 +687,342 @@ __global__ void __launch_bounds__(kTile, 2) k2_wave_f64(const Knot* __restrict__
         antenna_fixed<double>(g, cb, sb, scale, F);
       }
       double sph, cph, s2g, c2g, sa, ca;
-      sincos2pi_tab(fph, ex, sph, cph);
-      sincos2pi_tab(fgm, ex, s2g, c2g);
-      sincos2pi_tab(fal, ex, sa, ca);
+      sincos2pi_tab(fph, g_exp512, sph, cph);
+      sincos2pi_tab(fgm, g_exp512, s2g, c2g);
+      sincos2pi_tab(fal, g_exp512, sa, ca);
       double hI, hII;
       channels(g, cph, sph, c2g, s2g, ca, sa, A, (double)r * inv_span, bq, n_max, F, hI, hII);
       out = make_double2(hI, hII);
     }
-    z[(int64_t)wk * n + j] = out;
+    z[j] = out;
+  }
+}
+
+// ------------------------------------------- the same in fixed point (FP64)
+// Phase of one knot interval in fixed point: base + inc tau (Q64, mod 1) plus
+// s^2 (c2 + c3 s), s = tau / K_s, c2 in Q61 and c3 in Q62.
+struct PhX {
+  fx::u64 base;
+  fx::i64 inc, c2, c3;
+};
+struct IvX {
+  PhX ph, gm, al;
+};
+
+// false when the correction polynomial is outside its fixed-point range
+__device__ __forceinline__ bool phase_fixed(const double c[4], int ks, PhX& o) {
+  o.base = to_q64(c[0]);
+  o.inc = to_q64s(c[1] / ks);
+  o.c2 = llrint(c[2] * 0x1p61);
+  o.c3 = llrint(c[3] * 0x1p62);
+  return fabs(c[0]) < 1e9 && fabs(c[1]) < 1e9 && fabs(c[2]) < 1.0 && fabs(c[3]) < 1.0;   // (false for NaN)
+}
+
+// tau in [0, K_s), s31 = 2^31 tau / K_s
+__device__ __forceinline__ fx::u64 phase_at(const PhX& v, int tau, int s31) {
+  fx::i64 c = v.c2 + fx::mul31(v.c3, s31);      // Q61
+  c = fx::mul31(fx::mul31(c, s31), s31);        // Q59
+  return v.base + (fx::u64)tau * (fx::u64)v.inc + ((fx::u64)c << 5);
+}
+
+// Harmonic coefficients of a segment in fixed point: the quadratics
+// q0 + rho (q1 + rho q2) of a_n, b_n, c_n in rho = r/1024 (r: sample offset),
+// each times 2^k split as 2^27 h + l (0 <= l < 2^27), or q2 in h alone; signed
+// for the recurrence of harmonics_fixed.
+struct __align__(16) HarmX {
+  int4 a, b, c;   // (h0, l0, h1, l1)
+  int h2[4], l2[4];
+};
+
+// Block exponents of the coefficients and the shifts that align the sums.
+// S0, S1, S2: sums over harmonics and quantities of |q0|, |q1|, |q2|.  Every
+// accumulator of harmonics_fixed stays below 2^63: sum |q0| 2^k0 < 2^56,
+// sum |q1| 2^k1 < 2^50, sum |q2| 2^k2 < 2^29 (one word) or 2^51.  One word
+// (30 bits) rounds the sums by 2^-31 S2: taken where that is below 2^-54 S0,
+// as it is on all of an inspiral but its last hours.
+struct HarmScale {
+  int k0, k1, k2, sh1, sh2, two;
+};
+FX_HD HarmScale harm_scale(float S0, float S1, float S2) {
+  S0 = fmaxf(S0, 1e-20f);
+  S1 = fmaxf(fmaxf(S1, S2), S0 * 0x1p-24f);
+  S2 = fmaxf(S2, S1 * 0x1p-24f);
+  S0 = fmaxf(S0, 128.f * S1);
+  HarmScale o;
+  const int e0 = ilogbf(S0), e1 = ilogbf(S1), e2 = ilogbf(S2);
+  o.k0 = 55 - e0;
+  o.k1 = 49 - e1;
+  o.two = S2 > S0 * 0x1p-23f;
+  o.k2 = (o.two ? 50 : 28) - e2;
+  o.sh1 = o.k1 - o.k0 - 1;                      // in [0, 18]
+  o.sh2 = o.k2 - o.k1 + (o.two ? -1 : 23);      // in [0, 27]
+  return o;
+}
+
+// exact 2^k as a double, |k| < 1000
+__device__ __forceinline__ double pow2d(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
+
+// C = sum_n a_n cos(n Phi), S = sum_n b_n sin(n Phi), R = sum_n c_n cos(n Phi)
+// in units of 2^-(6 + k0) at sample offset r of the segment; cs: cos, sin of
+// Phi in Q62.
+//
+// d_n = +-cos(n Phi) follows d_{n+1} = -+ T d_n + d_{n-1}, T = 2 cos Phi (the
+// minus for odd n; signs + + - - over n mod 4, which the coefficients carry),
+// in Q59 -- the previous value is then the addend of the first multiply-add
+// and the product needs no shift.  Rounding per step ~2^-59, against ~2^-54 in
+// double.  Per harmonic 8 multiply-adds advance cosine and sine, 9 add the
+// constant, 9 the linear and 3 the quadratic coefficients (which are ~2^-9 and
+// ~2^-20 of the constant ones, so q2 mostly keeps one word, else kTwo): 29
+// multiply-adds and 8 others, ~145 cycles a warp, for 11 FP64 instructions
+// (836 cycles).
+template <bool kTwo>
+FX_HD void harmonics_fixed(fx::Trig cs, int r, const HarmX* __restrict__ hx, int n_max, int sh1,
+                                                int sh2, fx::i64& C, fx::i64& S, fx::i64& R) {
+  using namespace fx;
+  const Op tp = op(cs.c), tm = op(-cs.c);   // 2 cos Phi and its negative, Q61
+  i64 c0 = (i64)1 << 59, s0 = 0, c1 = cs.c >> 3, s1 = cs.s >> 3;
+  i64 h0[3] = {0, 0, 0}, x0[3] = {0, 0, 0}, h1[3] = {0, 0, 0}, x1[3] = {0, 0, 0}, h2[3] = {0, 0, 0},
+      x2[3] = {0, 0, 0};
+  auto acc = [&](int q, int4 k, int kh, int kl, int vh, int vl) {
+    h0[q] = wide(k.x, vh, h0[q]);
+    x0[q] = wide(k.x, vl, x0[q]);
+    x0[q] = wide(k.y, vh, x0[q]);
+    h1[q] = wide(k.z, vh, h1[q]);
+    x1[q] = wide(k.z, vl, x1[q]);
+    x1[q] = wide(k.w, vh, x1[q]);
+    h2[q] = wide(kh, vh, h2[q]);
+    if (kTwo) {
+      x2[q] = wide(kh, vl, x2[q]);
+      x2[q] = wide(kl, vh, x2[q]);
+    }
+  };
+  // one harmonic: adds it to the sums; (p0, p1) -> the next value in p0
+  auto step = [&](const HarmX& k, Op T, i64& cp, i64 cn, i64& sp, i64 sn) {
+    const i64 cv = cn << 3, sv = sn << 3;   // Q62
+    const int ch = hi(cv), sh = hi(sv);
+    acc(0, k.a, k.h2[0], k.l2[0], ch, lo27(cv));
+    acc(1, k.b, k.h2[1], k.l2[1], sh, lo27(sv));
+    acc(2, k.c, k.h2[2], k.l2[2], ch, lo27(cv));
+    Sum nc(cp), ns(sp);
+    nc.add(T, Op{ch, lo31(cv)});
+    ns.add(T, Op{sh, lo31(sv)});
+    cp = nc.get();
+    sp = ns.get();
+  };
+  int n = 0;
+#pragma unroll 1
+  for (; n + 1 < n_max; n += 2) {
+    step(hx[n], tm, c0, c1, s0, s1);
+    step(hx[n + 1], tp, c1, c0, s1, s0);
+  }
+  if (n < n_max) step(hx[n], tm, c0, c1, s0, s1);
+  const int rho = r << 21;   // 2^31 r / 1024
+  i64 v[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const i64 w2 = kTwo ? (h2[q] << 3) + (x2[q] >> 24) : h2[q];
+    const i64 w1 = (h1[q] << 3) + (x1[q] >> 24) + (mul31(w2, rho) >> sh2);
+    v[q] = (h0[q] << 3) + (x0[q] >> 24) + (mul31(w1, rho) >> sh1);
+  }
+  C = v[0];
+  S = v[1];
+  R = v[2];
+}
+
+// Geometry constants of the response, Q62 (spS, sqS: Q60)
+struct GeoX {
+  fx::Op pe1, pe2n, qe1, qe2n, cpe1, cpe2, cqe1, cqe2;
+  fx::i64 spSn, sqSn;
+};
+
+// response() in fixed point: H+ and Hx in units of 2^-(2 + k0) from the sums
+// in units of 2^-(6 + k0).  |z_1|, |z_2| <= 1 (projections of unit vectors).
+FX_HD void response_fixed(const GeoX& g, fx::Trig gm, fx::Trig al, fx::i64 Cs, fx::i64 Ss,
+                                               fx::i64 Rs, fx::i64& Hp, fx::i64& Hx) {
+  using namespace fx;
+  const Op ca = op(al.c), sa = op(al.s);
+  auto proj = [&](Op x, Op kx, Op y, Op ky, i64 add) {   // Q60 sums, returned in Q62
+    Sum s(add);
+    s.add(x, kx);
+    s.add(y, ky);
+    return s.get() << 2;
+  };
+  const i64 z1r = proj(sa, g.pe1, ca, g.pe2n, 0), z1i = proj(sa, g.qe1, ca, g.qe2n, 0);
+  const i64 z2r = proj(ca, g.cpe1, sa, g.cpe2, g.spSn), z2i = proj(ca, g.cqe1, sa, g.cqe2, g.sqSn);
+  i64 a, b, y;   // A = 1: (Rs + X)/4, (Rs - X)/4, 2 Y/4
+  {
+    const Op c = op(Cs), s = op(Ss), g2c = op(gm.c);
+    Sum X, Y;
+    X.add(c, g2c);
+    X.add(s, op(-gm.s));
+    Y.add(c, op(gm.s));
+    Y.add(s, g2c);
+    const i64 x = X.get();
+    a = (Rs >> 2) + x;
+    b = (Rs >> 2) - x;
+    y = Y.get() << 1;
+  }
+  const Op z1ro = op(z1r), z1io = op(z1i), z2ro = op(z2r), z2io = op(z2i), ao = op(a), bo = op(b), yo = op(y);
+  Sum p, q, c;
+  p.add(ao, op(mul(op(z1r - z1i), op(z1r + z1i)) << 2));
+  p.add(bo, op(mul(op(z2r - z2i), op(z2r + z2i)) << 2));
+  q.add(yo, op((mul(z1ro, z2ro) - mul(z1io, z2io)) << 2));
+  Hp = p.get() + q.get();
+  c.add(z1ro, z2io);
+  c.add(z1io, z2ro);
+  Sum u, w;
+  u.add(ao, op(mul(z1ro, z1io) << 3));
+  u.add(bo, op(mul(z2ro, z2io) << 3));
+  w.add(yo, op(c.get() << 2));
+  Hx = u.get() + w.get();
+}
+
+// What bounds it: FP64 issue (1 warp instruction per 76 cycles).  In double a
+// sample takes 333 FP64 instructions at n_max = 20: 156.3 ms for 128 walkers x
+// 2^21 samples, 6.73 ms for 8 walkers x 2^21 at n_max = 10.  Here the phases,
+// their sines and cosines, the harmonic sums and the response run in 64-bit
+// fixed point on the integer pipe (~4200 cycles a warp at n_max = 20), and
+// only the slowly varying factors (x^(2/3), the patterns) stay in double,
+// beside them: 24 FP64 instructions.  56.7 and 2.59 ms.
+__global__ void __launch_bounds__(kTile, 2) k2_wave_f64(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
+                                                        int64_t n, double dt, double t0, int ks, int n_max,
+                                                        double2* __restrict__ z, int unit_scale, int exact_f,
+                                                        const double* __restrict__ bc, const double* __restrict__ ifact,
+                                                        const double* __restrict__ lisa) {
+  constexpr int kTiles = kSegF / kTile;
+  __shared__ IvD iv[kSegF / 64];
+  __shared__ IvX ivx[kSegF / 64];
+  __shared__ double bnode[3 * 32 * 3];
+  __shared__ double bq[32 * 9];
+  __shared__ HarmX hx[32];
+  __shared__ HarmScale hsc;
+  __shared__ double fn[kTiles][4][4];   // the four patterns at the four fit nodes of each tile
+  __shared__ double fq[kTiles][4][4];   // their cubics in (t mod 256) / 256
+  __shared__ fx::Trig ex[fx::kTrigLen];
+  __shared__ Geo<double> g;
+  __shared__ GeoX gx;
+  __shared__ int fixed_bad;
+  const int wk = blockIdx.y;
+  const WalkerC& C = wcs[wk];
+  const int64_t nk = n / ks;
+  const Knot* kn = knots + (int64_t)wk * (nk + 1);
+  const int64_t j0 = (int64_t)blockIdx.x * kSegF;
+  const int64_t kfirst = j0 / ks;
+  const int ni = ks >= kSegF ? 1 : kSegF / ks;
+  const int t = threadIdx.x;
+  const double h = (double)ks * dt;
+  const double scale = unit_scale ? C.gd.amp_scale : 1.0;
+  z += (int64_t)wk * n;
+  const int64_t jplunge = C.j_plunge;
+  if (jplunge <= j0) {   // nothing left of the inspiral
+    for (int r = t; r < kSegF; r += kTile) z[j0 + r] = make_double2(0.0, 0.0);
+    return;
+  }
+  if (t == 0) fixed_bad = exact_f;
+  __syncthreads();
+  if (t < ni) {
+    build_iv(kn[kfirst + t], kn[kfirst + t + 1], h, iv[t]);
+    const bool ok0 = phase_fixed(iv[t].ph, ks, ivx[t].ph), ok1 = phase_fixed(iv[t].gm, ks, ivx[t].gm),
+               ok2 = phase_fixed(iv[t].al, ks, ivx[t].al);
+    if (!(ok0 && ok1 && ok2)) fixed_bad = 1;
+  }
+  if (t >= 224 && t < 224 + 4 * kTiles && !exact_f) {   // node q of tile tt
+    const int i = t - 224, tt = i / 4, q = i % 4;
+    const double* L = lisa + ((int64_t)blockIdx.x * kTiles + tt) * 8 + 2 * q;
+    antenna_fixed<double>(C.gd, L[0], L[1], scale, fn[tt][q]);
+  }
+  if (t >= 160 && t < 170) {   // geometry constants, one per thread
+    const Geo<double>& G = C.gd;
+    const int i = t - 160;
+    const double v = i == 0 ? G.pe1 : i == 1 ? -G.pe2 : i == 2 ? G.qe1 : i == 3 ? -G.qe2 : i == 4 ? G.cpe1
+                   : i == 5 ? G.cpe2 : i == 6 ? G.cqe1 : i == 7 ? G.cqe2 : i == 8 ? -G.spS : -G.sqS;
+    if (!(fabs(v) < 1.0000001)) fixed_bad = 1;
+    if (i < 8) (&gx.pe1)[i] = fx::op(llrint(v * 0x1p62));
+    else (&gx.spSn)[i - 8] = llrint(v * 0x1p60);
+    if (i == 0) g = G;
+  }
+  for (int i = t; i < fx::kTrigLen; i += kTile) ex[i] = g_trig[i];
+  __syncthreads();
+  const int span = tile_span(j0, jplunge, kSegF);
+  tile_harmonics<double, IvD>(iv, ni, j0, kfirst, ks, n_max, span, bnode, bq, bc, ifact);
+  __syncthreads();
+  if (t < 32) {   // block exponents
+    const float rs = (float)kSegF / (float)span;
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    if (t < n_max)
+      for (int f = 0; f < 3; ++f) {
+        const double* b = bq + 9 * t + 3 * f;
+        s0 += fabsf((float)b[0]);
+        s1 += fabsf((float)b[1]) * rs;
+        s2 += fabsf((float)b[2]) * (rs * rs);
+      }
+    for (int off = 16; off > 0; off >>= 1) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+    }
+    if (t == 0) {
+      hsc = harm_scale(1.0001f * s0, 1.0001f * s1, 1.0001f * s2);
+      // amplitudes that move by more than 1/32 of their sum over the segment
+      // (the unit of q0 follows 128 S1) or are not finite: in double
+      if (!(s0 < 1e12f && 32.f * s1 < s0 && s2 < s0)) fixed_bad = 1;
+    }
+  }
+  __syncthreads();
+  const bool fixed = !fixed_bad;
+  if (fixed) {
+    const double rs = (double)kSegF / (double)span;
+    for (int i = t; i < 9 * n_max; i += kTile) {
+      const int m = i / 9, f = (i % 9) / 3, p = i % 3;
+      double v = bq[i];
+      if ((m + 1) & 2) v = -v;   // the signs of the recurrence
+      v *= p == 0 ? pow2d(hsc.k0) : p == 1 ? pow2d(hsc.k1) * rs : pow2d(hsc.k2) * (rs * rs);
+      const fx::i64 q = llrint(v);
+      int* o = reinterpret_cast<int*>(hx + m);
+      int* oh = p < 2 ? o + 4 * f + 2 * p : hx[m].h2 + f;
+      int* ol = p < 2 ? oh + 1 : hx[m].l2 + f;
+      const bool one = p == 2 && !hsc.two;
+      *oh = (int)(one ? q : q >> 27);
+      *ol = one ? 0 : (int)(q & ((1 << 27) - 1));
+    }
+  }
+  if (t >= 224 && t < 224 + 4 * kTiles && !exact_f) {   // pattern q of tile tt, in the sums' unit
+    const int i = t - 224, tt = i / 4, q = i % 4;
+    const double u = fixed ? pow2d(-2 - hsc.k0) : 1.0;
+    fit_cubic4<double>(u * fn[tt][0][q], u * fn[tt][1][q], u * fn[tt][2][q], u * fn[tt][3][q], fq[tt][q]);
+  }
+  __syncthreads();
+  if (!fixed) {
+    wave_samples_f64(iv, bq, fq, g, j0, kfirst, jplunge, span, dt, t0, ks, n_max, scale, exact_f, z);
+    return;
+  }
+  const int lks = __ffs(ks) - 1;   // ks: a power of two
+  const double so = (double)t * (1.0 / kTile);
+  const double inv_ks = 1.0 / (double)ks;
+#pragma unroll 1
+  for (int tt = 0; tt < kTiles; ++tt) {
+    const int r = tt * kTile + t;   // offset in the segment
+    const int64_t j = j0 + r;
+    double2 out = make_double2(0.0, 0.0);
+    if (j < jplunge) {
+      const int ki = ks >= kSegF ? 0 : r >> lks;
+      const int tau = ks >= kSegF ? r : r & (ks - 1);
+      const int s31 = tau << (31 - lks);
+      const IvX& v = ivx[ki];
+      fx::i64 Cs, Ss, Rs, Hp, Hx;
+      const fx::Trig ph = fx::sincos_cycles(phase_at(v.ph, tau, s31), ex);
+      if (hsc.two) harmonics_fixed<true>(ph, r, hx, n_max, hsc.sh1, hsc.sh2, Cs, Ss, Rs);
+      else harmonics_fixed<false>(ph, r, hx, n_max, hsc.sh1, hsc.sh2, Cs, Ss, Rs);
+      response_fixed(gx, fx::sincos_cycles(phase_at(v.gm, tau, s31), ex),
+                     fx::sincos_cycles(phase_at(v.al, tau, s31), ex), Cs, Ss, Rs, Hp, Hx);
+      const double A = poly3<double>(iv[ki].am, (double)tau * inv_ks);
+      double F[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) F[q] = cubic_at<double>(fq[tt][q], so);
+      const double hp = (double)Hp, hc = (double)Hx;
+      out = make_double2(A * (F[0] * hp + F[1] * hc), A * (F[2] * hp + F[3] * hc));
+    }
+    z[j] = out;
   }
 }
 
