@@ -310,7 +310,7 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   const double hh_scale = f32 ? 1.0 / ds->w_scale : 1.0;
   // steps S5-S7 of walkers [j0, j0 + gw), whose series start at zg
   auto passes = [&](int j0, int gw, char* zg, cudaStream_t st) {
-    { KTimer t(pf, EMRI_K_FFT1, st); launch_fft_pass1(zg, gw, p, f32, -1, ctx->tw, st); }
+    { KTimer t(pf, EMRI_K_FFT1, st); launch_fft_pass1(zg, zg, gw, p, f32, -1, ctx->tw, st); }
     {
       KTimer t(pf, EMRI_K_FFT2_IP, st);
       launch_fft_pass2_ip(zg, gw, p, f32, ctx->tw, b.wc + j0, b.dtab + (size_t)j0 * p.n1 * cs,
@@ -692,7 +692,7 @@ extern "C" int emri_dataset_create(emri_ctx* ctx, const emri_grid* grid, const v
       double* d2 = (double*)scratch;   // [2][n] doubles fit in the n-complex scratch
       if ((e = cudaMemcpyAsync(d2, data, (size_t)n * 16, cudaMemcpyDefault, s)) != cudaSuccess) break;
       launch_pack_time_series(d2, n, dnat, s);
-      launch_fft_pass1(dnat, 1, ds->plan, false, -1, ctx->tw, s);
+      launch_fft_pass1(dnat, dnat, 1, ds->plan, false, -1, ctx->tw, s);
       launch_fft_pass2_store(dnat, scratch, 1, ds->plan, false, -1, ctx->tw, s);
       if ((e = cudaMemcpyAsync(dnat, scratch, (size_t)n * 16, cudaMemcpyDeviceToDevice, s)) != cudaSuccess) break;
     }
@@ -853,18 +853,16 @@ extern "C" int emri_fft_batch(emri_ctx* ctx, void* z, int64_t n, int batch, int 
   if ((rc = ctx->ws.reserve(ctx, (size_t)chunk * n * cs + 256, s))) return rc;
   ctx->ws.acquire(s);
   int64_t nl = 0;
-  cudaError_t e = cudaSuccess;
-  for (int b0 = 0; b0 < batch && e == cudaSuccess; b0 += chunk) {
+  for (int b0 = 0; b0 < batch; b0 += chunk) {
     const int bb = std::min(chunk, batch - b0);
     char* zb = (char*)z + (size_t)b0 * n * cs;
-    launch_fft_pass1(zb, bb, p, f32, direction, ctx->tw, s);
-    launch_fft_pass2_store(zb, ctx->ws.ptr, bb, p, f32, direction, ctx->tw, s);
-    e = cudaMemcpyAsync(zb, ctx->ws.ptr, (size_t)bb * n * cs, cudaMemcpyDeviceToDevice, s);
+    launch_fft_pass1(zb, ctx->ws.ptr, bb, p, f32, direction, ctx->tw, s);
+    launch_fft_pass2_store(ctx->ws.ptr, zb, bb, p, f32, direction, ctx->tw, s);
     nl += 2;
   }
   ctx->ws.release(s);
   ctx->launches += nl;
-  if (e == cudaSuccess) e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "fft launch");
   return EMRI_OK;
 }

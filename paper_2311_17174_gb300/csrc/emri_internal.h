@@ -63,6 +63,7 @@ int upload_exp512();
 
 void launch_prologue(const double* theta, int64_t ld, int w, int64_t n, double dt, const OptsN& o,
                      const double* gl, WalkerC* out, cudaStream_t s);
+// (FP64 tab with n1 >= 256: (cos.h, cos.l, sin.h, sin.l) in Q62, four ints)
 // tab[w][n1] = exp(-2 pi i frac(n2 k1 r)), rtab[w][n2] = exp(-2 pi i frac(k2 r))
 void launch_delay_table(const WalkerC* wc, int w, int n1, int n2, bool fp32, void* tab, void* rtab, cudaStream_t s);
 void launch_prologue_export(const WalkerC* wc, int w, double* out, cudaStream_t s);
@@ -92,8 +93,8 @@ inline const double2* lisa_knots(const double* tab, int64_t n) { return (const d
 void launch_lisa(int64_t n, int ks, double t0, double dt, double* tab, cudaStream_t s);
 constexpr size_t kIvMBytes = 104;
 
-// FFT pass 1 (columns, in place, with the inter-pass twiddle); sign -1 forward, +1 inverse
-void launch_fft_pass1(void* z, int batch, const FftPlan& p, bool fp32, int sign, const Twiddles& t,
+// FFT pass 1 (columns, with the inter-pass twiddle; out may be z); sign -1 forward, +1 inverse
+void launch_fft_pass1(const void* z, void* out, int batch, const FftPlan& p, bool fp32, int sign, const Twiddles& t,
                       cudaStream_t s);
 // FFT pass 2 to natural order into out (out-of-place)
 void launch_fft_pass2_store(const void* y, void* out, int batch, const FftPlan& p, bool fp32, int sign,

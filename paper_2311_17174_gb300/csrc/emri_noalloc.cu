@@ -8,7 +8,7 @@
 // callers cannot create an emri_ctx (its creation allocates tables and
 // workspaces), so this entry point takes no context at all.
 //
-// How: the FFT's second pass writes out of place into scratch memory.  That
+// How: the FFT's first pass writes to scratch memory, the second one back.  That
 // scratch (32 MiB, at least one whole sequence: 2^21 double2 or 2^22 float2
 // values, and several sequences per pass when they are shorter) and the
 // twiddle tables the passes read are file-scope static device arrays of
@@ -122,10 +122,8 @@ extern "C" int emri_fft_batch_noalloc(void* z, int64_t n, int batch, int precisi
   for (int b0 = 0; b0 < batch; b0 += chunk) {
     const int bb = batch - b0 < chunk ? batch - b0 : chunk;
     char* zb = (char*)z + (size_t)b0 * n * cs;
-    launch_fft_pass1(zb, bb, p, f32, direction, st->tw, s);
-    launch_fft_pass2_store(zb, st->scratch, bb, p, f32, direction, st->tw, s);
-    e = cudaMemcpyAsync(zb, st->scratch, (size_t)bb * n * cs, cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return cuda_err(e, "no-alloc FFT copy-back");
+    launch_fft_pass1(zb, st->scratch, bb, p, f32, direction, st->tw, s);
+    launch_fft_pass2_store(st->scratch, zb, bb, p, f32, direction, st->tw, s);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "no-alloc FFT launch");

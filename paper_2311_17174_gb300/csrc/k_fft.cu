@@ -4,11 +4,13 @@
 //
 // n = n1 * n2 (four-step): element j = j1 + n1 j2, bin k = k2 + n2 k1.
 //  pass 1: for each column j1, the n2-point DFT over j2, times the twiddle
-//          exp(-2 pi i j1 k2 / n), written back in place (position j1 + n1 k2);
+//          exp(-2 pi i j1 k2 / n), written to position j1 + n1 k2 (in place, or
+//          to another buffer);
 //  pass 2: for each row k2, the n1-point DFT over j1 gives bins k2 + n2 k1.
-// Both passes are shared-memory Stockham FFTs, one CTA per column group /
-// row: radix-4 stages (one radix-2 stage when log2 of the length is odd) in
-// FP64, radix-8 stages (then one radix-4 or radix-2) in FP32.
+// Both passes are Stockham FFTs, one CTA per column group / row, radix 8 (then
+// one radix-4 or radix-2 stage): FP64 of 256 points or more in 64-bit fixed
+// point (fft_fixed.cuh), FP32 in float, in registers or shared memory; shorter
+// FP64 transforms are radix 4 in shared memory.
 // The likelihood path never writes the spectrum: pass 2 multiplies each bin
 // by the GW-speed delay factor and accumulates
 //   sum_k w_k Re(conj(D_k) H_k e^{-2 pi i k_s r})  and  sum_k w_k |H_k|^2
@@ -21,6 +23,7 @@
 // read tc[i] = (cos, tan) of the same angles.
 #include "emri_common.cuh"
 #include "emri_internal.h"
+#include "fx64.cuh"
 
 namespace emri {
 
@@ -79,8 +82,11 @@ __global__ void k_twiddle_init(double2* ta64, double2* tb64, float2* ta32, float
   }
 }
 
+static void launch_fixed_twiddles(cudaStream_t s);
+
 void launch_twiddle_init(Twiddles t, cudaStream_t s) {
   k_twiddle_init<<<16, 256, 0, s>>>(t.ta64, t.tb64, t.ta32, t.tb32, t.tc64, t.tt32);
+  launch_fixed_twiddles(s);
 }
 
 // ----------------------------------------------------- complex helpers
@@ -609,13 +615,14 @@ __device__ __forceinline__ void last_stage(float2 (&v)[8], const float2* __restr
 // row-major (rows of NB contiguous elements), transformed along the rows
 // index, and written back in place with the inter-pass twiddle.
 template <typename C2, int LG, int NB>
-__global__ void __launch_bounds__(kFftThreads, sizeof(C2) == 8 ? 2 : 1) k3_pass1(C2* __restrict__ z, int64_t n, int n1, int sign, int shift22,
+__global__ void __launch_bounds__(kFftThreads, sizeof(C2) == 8 ? 2 : 1) k3_pass1(const C2* zin, C2* zout, int64_t n, int n1, int sign, int shift22,
                                                         const C2* __restrict__ ta, const C2* __restrict__ tb,
                                                         const C2* __restrict__ tf) {
   extern __shared__ __align__(16) unsigned char smraw[];
   C2* buf = reinterpret_cast<C2*>(smraw);
   constexpr int N2 = 1 << LG;
-  C2* zw = z + (int64_t)blockIdx.y * n;
+  const C2* zw = zin + (int64_t)blockIdx.y * n;
+  C2* zo = zout + (int64_t)blockIdx.y * n;
   const int j10 = blockIdx.x * NB;
   if constexpr (sizeof(C2) == 8) {
     // the tile's rows (NB * 8 bytes each) by cp.async: all of it in flight,
@@ -649,11 +656,12 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(C2) == 8 ? 2 : 1) k3_pass1
   for (int idx = threadIdx.x; idx < NB * N2; idx += kFftThreads, ++i) {
     const int k2 = idx / NB;
     w = (i & 3) == 0 ? twiddle22(ta, tb, (uint32_t)((j10 + c) * k2) << shift22, sign) : cmul(w, wstep);
-    zw[j10 + c + (int64_t)n1 * k2] = cmul(buf[idx], w);
+    zo[j10 + c + (int64_t)n1 * k2] = cmul(buf[idx], w);
   }
 }
 
 // --------------------------------------------------- pass 2, natural order
+// Rows of up to 128 points (FP64: fft_fixed.cuh from 256 on; FP32: below)
 template <typename C2, int LG>
 __global__ void __launch_bounds__(kPass2Threads, 2) k4_pass2_store(const C2* __restrict__ y, C2* __restrict__ out,
                                                                    int64_t n, int n2, int sign,
@@ -668,6 +676,49 @@ __global__ void __launch_bounds__(kPass2Threads, 2) k4_pass2_store(const C2* __r
   tile_fft<C2, LG, 1, kPass2Threads>(buf, sign, tf);
   C2* o = out + (int64_t)blockIdx.y * n;
   for (int k1 = threadIdx.x; k1 < N1; k1 += kPass2Threads) o[k2 + (int64_t)n2 * k1] = buf[k1];
+}
+
+// FP32, rows of 256 to 4096 points in registers (r8): NB adjacent rows a CTA,
+// so that the bins k2..k2 + NB - 1 of one k1, neighbours in the output, are
+// written together (NB = 4: whole 32-byte sectors; one row a CTA writes 8
+// bytes of each sector, and DRAM then reads the sector back).  The rows turn
+// over in shared memory on the way out.  75 inverse transforms of 2^20, with
+// pass 1 writing to the scratch buffer instead of a copy back at the end:
+// 1.43 -> 0.82 ms.  The inverse transform is the forward
+// one with Re and Im exchanged.
+template <int LG, int NB>
+__global__ void __launch_bounds__(NB * (1 << LG) / 8)
+    k4_pass2_store_r8(const float2* __restrict__ y, float2* __restrict__ out, int64_t n, int n2, int sign,
+                      const float2* __restrict__ tt) {
+  constexpr int N1 = 1 << LG, T = N1 / 8, PAD = N1 + N1 / 16;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float2* sm = reinterpret_cast<float2*>(smraw);
+  const int c = threadIdx.x / T, t = threadIdx.x % T;
+  const float2* row = y + (int64_t)blockIdx.y * n + (int64_t)N1 * (blockIdx.x * NB + c);
+  float2 v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float2 u = row[t + q * T];
+    v[q] = sign > 0 ? make_float2(u.y, u.x) : u;
+  }
+  r8::stages8<LG, 0>(v, sm + c * PAD, tt, t);
+  r8::last_stage<LG>(v, tt, t);
+  float2* o = out + (int64_t)blockIdx.y * n + blockIdx.x * NB;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    if (sign > 0) v[q] = make_float2(v[q].y, v[q].x);
+    if (NB == 1) o[(int64_t)n2 * (t + q * T)] = v[q];
+  }
+  if constexpr (NB > 1) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sm[c * PAD + r8::pad16(t + q * T)] = v[q];
+    __syncthreads();
+    for (int i = threadIdx.x; i < NB * N1; i += NB * T) {
+      const int r = i % NB, k1 = i / NB;
+      o[r + (int64_t)n2 * k1] = sm[r * PAD + r8::pad16(k1)];
+    }
+  }
 }
 
 // -------------------------------------------- pass 2 fused with the IP
@@ -954,6 +1005,8 @@ __global__ void __launch_bounds__((1 << LG) / 8)
   }
 }
 
+#include "fft_fixed.cuh"
+
 template <int LG>
 constexpr size_t r8_smem() {
   return (size_t)((1 << LG) + (1 << LG) / 16) * sizeof(float2);
@@ -1048,26 +1101,26 @@ template <typename C2>
 static size_t csize() { return sizeof(C2); }
 
 template <typename C2, int NB, int LG>
-static void pass1_inst(C2* z, int batch, const FftPlan& p, int sign, int shift, const C2* ta, const C2* tb,
+static void pass1_inst(const C2* z, C2* out, int batch, const FftPlan& p, int sign, int shift, const C2* ta, const C2* tb,
                        const C2* tf, cudaStream_t s) {
   dim3 g(p.n1 / NB, batch);
-  k3_pass1<C2, LG, NB><<<g, kFftThreads, (size_t)NB * (1 << LG) * sizeof(C2), s>>>(z, p.n, p.n1, sign, shift, ta, tb,
+  k3_pass1<C2, LG, NB><<<g, kFftThreads, (size_t)NB * (1 << LG) * sizeof(C2), s>>>(z, out, p.n, p.n1, sign, shift, ta, tb,
                                                                                     tf);
 }
 
 template <typename C2, int NB>
-static void pass1_dispatch(C2* z, int batch, const FftPlan& p, int sign, const C2* ta, const C2* tb, const C2* tf,
+static void pass1_dispatch(const C2* z, C2* out, int batch, const FftPlan& p, int sign, const C2* ta, const C2* tb, const C2* tf,
                            cudaStream_t s) {
   const int shift = 22 - p.log2n;
   int lg = 0;
   while ((1 << lg) < p.n2) ++lg;
-  switch (lg) {
-    case 5: pass1_inst<C2, NB, 5>(z, batch, p, sign, shift, ta, tb, tf, s); break;
-    case 6: pass1_inst<C2, NB, 6>(z, batch, p, sign, shift, ta, tb, tf, s); break;
-    case 7: pass1_inst<C2, NB, 7>(z, batch, p, sign, shift, ta, tb, tf, s); break;
-    case 8: pass1_inst<C2, NB, 8>(z, batch, p, sign, shift, ta, tb, tf, s); break;
-    case 9: pass1_inst<C2, NB, 9>(z, batch, p, sign, shift, ta, tb, tf, s); break;
-    default: pass1_inst<C2, NB, 10>(z, batch, p, sign, shift, ta, tb, tf, s); break;
+  if (lg == 5) pass1_inst<C2, NB, 5>(z, out, batch, p, sign, shift, ta, tb, tf, s);
+  if (lg == 6) pass1_inst<C2, NB, 6>(z, out, batch, p, sign, shift, ta, tb, tf, s);
+  if (lg == 7) pass1_inst<C2, NB, 7>(z, out, batch, p, sign, shift, ta, tb, tf, s);
+  if constexpr (sizeof(C2) == sizeof(float2)) {   // FP64 columns of 256 points and more: pass1_fixed
+    if (lg == 8) pass1_inst<C2, NB, 8>(z, out, batch, p, sign, shift, ta, tb, tf, s);
+    if (lg == 9) pass1_inst<C2, NB, 9>(z, out, batch, p, sign, shift, ta, tb, tf, s);
+    if (lg >= 10) pass1_inst<C2, NB, 10>(z, out, batch, p, sign, shift, ta, tb, tf, s);
   }
 }
 
@@ -1078,27 +1131,31 @@ static int log2i(int v) {
 }
 
 
-void launch_fft_pass1(void* z, int batch, const FftPlan& p, bool fp32, int sign, const Twiddles& t,
+static void launch_fixed_twiddles(cudaStream_t s) { fxfft::k_init<<<16, 256, 0, s>>>(); }
+
+// FP64 columns of 256, 512, 1024 points: fixed point, 256 threads a CTA
+template <int LG>
+static void pass1_fixed(const double2* z, double2* out, int batch, const FftPlan& p, int sign, const Twiddles& t, cudaStream_t s) {
+  constexpr int NB = 2048 >> LG;
+  using F = fxfft::Cfg<LG, NB>;
+  fxfft::k3_pass1_fixed<LG, NB><<<dim3(p.n1 / NB, batch), F::kThreads, F::kSmem, s>>>(
+      z, out, p.n, p.n1, sign, 22 - p.log2n, t.ta64, t.tb64, t.tc64);
+}
+
+void launch_fft_pass1(const void* z, void* out, int batch, const FftPlan& p, bool fp32, int sign, const Twiddles& t,
                       cudaStream_t s) {
   if (batch <= 0) return;
   if (fp32)
-    pass1_dispatch<float2, FftCfg<float2>::kCols>((float2*)z, batch, p, sign, t.ta32, t.tb32, t.ta32, s);
+    pass1_dispatch<float2, FftCfg<float2>::kCols>((const float2*)z, (float2*)out, batch, p, sign, t.ta32, t.tb32, t.ta32, s);
+  else if (p.n2 >= 1024)
+    pass1_fixed<10>((const double2*)z, (double2*)out, batch, p, sign, t, s);
+  else if (p.n2 == 512)
+    pass1_fixed<9>((const double2*)z, (double2*)out, batch, p, sign, t, s);
+  else if (p.n2 == 256)
+    pass1_fixed<8>((const double2*)z, (double2*)out, batch, p, sign, t, s);
   else
-    pass1_dispatch<double2, FftCfg<double2>::kCols>((double2*)z, batch, p, sign, t.ta64, t.tb64, t.tc64, s);
+    pass1_dispatch<double2, FftCfg<double2>::kCols>((const double2*)z, (double2*)out, batch, p, sign, t.ta64, t.tb64, t.tc64, s);
 }
-
-#define EMRI_LG_SWITCH(lg, CALL)  \
-  switch (lg) {                   \
-    case 5: CALL(5); break;       \
-    case 6: CALL(6); break;       \
-    case 7: CALL(7); break;       \
-    case 8: CALL(8); break;       \
-    case 9: CALL(9); break;       \
-    case 10: CALL(10); break;     \
-    case 11: CALL(11); break;     \
-    default: CALL(12); break;     \
-  }
-
 
 void launch_fft_pass2_store(const void* y, void* out, int batch, const FftPlan& p, bool fp32, int sign,
                             const Twiddles& t, cudaStream_t s) {
@@ -1108,12 +1165,36 @@ void launch_fft_pass2_store(const void* y, void* out, int batch, const FftPlan& 
   if (fp32) {
 #define CALL32(L) k4_pass2_store<float2, L><<<g, kPass2Threads, p.n1 * sizeof(float2), s>>>( \
       (const float2*)y, (float2*)out, p.n, p.n2, sign, t.ta32)
-    EMRI_LG_SWITCH(lg, CALL32)
+#define CALLR8(L, NB) k4_pass2_store_r8<L, NB><<<dim3(p.n2 / NB, batch), NB * (1 << L) / 8, NB * r8_smem<L>(), s>>>( \
+      (const float2*)y, (float2*)out, p.n, p.n2, sign, t.tt32)
+    switch (lg) {
+      case 5: CALL32(5); break;
+      case 6: CALL32(6); break;
+      case 7: CALL32(7); break;
+      case 8: CALLR8(8, 8); break;
+      case 9: CALLR8(9, 4); break;
+      case 10: CALLR8(10, 4); break;
+      case 11: CALLR8(11, 4); break;
+      default: CALLR8(12, 2); break;
+    }
+#undef CALLR8
 #undef CALL32
   } else {
 #define CALL64(L) k4_pass2_store<double2, L><<<g, kPass2Threads, p.n1 * sizeof(double2), s>>>( \
       (const double2*)y, (double2*)out, p.n, p.n2, sign, t.tc64)
-    EMRI_LG_SWITCH(lg, CALL64)
+#define CALLX(L, NB) fxfft::k4_pass2_store_fixed<L, NB><<<dim3(p.n2 / NB, batch), fxfft::Cfg<L, NB>::kThreads, \
+      fxfft::Cfg<L, NB>::kSmem, s>>>((const double2*)y, (double2*)out, p.n, p.n2, sign, t.tc64)
+    switch (lg) {
+      case 5: CALL64(5); break;
+      case 6: CALL64(6); break;
+      case 7: CALL64(7); break;
+      case 8: CALLX(8, 2); break;
+      case 9: CALLX(9, 2); break;
+      case 10: CALLX(10, 2); break;
+      case 11: CALLX(11, 2); break;
+      default: CALLX(12, 1); break;   // 512 threads a row
+    }
+#undef CALLX
 #undef CALL64
   }
 }
@@ -1140,13 +1221,30 @@ static void pass2_ip_dispatch(const void* y, int w, const FftPlan& p, bool fp32,
 #define CALLI32(L) k4_pass2_ip<float2, float, AccF, L, FD><<<g, kPass2Threads, P2Smem<float2, float, L>::bytes(), s>>>( \
       (const float2*)y, p.n, p.n2, t.ta32, wc, (const float2*)delay_tab, (const float2*)row_tab,                \
       (const float2*)data_perm, (const float*)wt_perm, partial, fd)
-    EMRI_LG_SWITCH(lg, CALLI32)
+    switch (lg) {
+      case 5: CALLI32(5); break;
+      case 6: CALLI32(6); break;
+      default: CALLI32(7); break;
+    }
 #undef CALLI32
   } else {
 #define CALLI64(L) k4_pass2_ip<double2, double, AccD, L, FD><<<g, kPass2Threads, P2Smem<double2, double, L>::bytes(), s>>>( \
       (const double2*)y, p.n, p.n2, t.tc64, wc, (const double2*)delay_tab, (const double2*)row_tab,                 \
       (const double2*)data_perm, (const double*)wt_perm, partial, fd)
-    EMRI_LG_SWITCH(lg, CALLI64)
+#define CALLX(L) fxfft::k4_pass2_ip_fixed<L, FD><<<g, fxfft::Cfg<L, 1>::kThreads, fxfft::Cfg<L, 1>::kSmem, s>>>(     \
+      (const double2*)y, p.n, p.n2, t.tc64, wc, (const int4*)delay_tab, (const double2*)row_tab,                    \
+      (const double2*)data_perm, (const double*)wt_perm, partial, fd)
+    switch (lg) {
+      case 5: CALLI64(5); break;
+      case 6: CALLI64(6); break;
+      case 7: CALLI64(7); break;
+      case 8: CALLX(8); break;
+      case 9: CALLX(9); break;
+      case 10: CALLX(10); break;
+      case 11: CALLX(11); break;
+      default: CALLX(12); break;
+    }
+#undef CALLX
 #undef CALLI64
   }
 }
@@ -1193,14 +1291,24 @@ static void raise(F f) {
 }
 
 void fft_set_smem_limits() {
-#define P1(L) raise(k3_pass1<double2, L, FftCfg<double2>::kCols>), raise(k3_pass1<float2, L, FftCfg<float2>::kCols>)
+#define P1(L) raise(k3_pass1<float2, L, FftCfg<float2>::kCols>)
   P1(5); P1(6); P1(7); P1(8); P1(9); P1(10);
 #undef P1
-#define P2(L) raise(k4_pass2_store<double2, L>), raise(k4_pass2_store<float2, L>), \
+  raise(k4_pass2_store<float2, 5>), raise(k4_pass2_store<float2, 6>), raise(k4_pass2_store<float2, 7>);
+  raise(k4_pass2_store_r8<8, 8>), raise(k4_pass2_store_r8<9, 4>), raise(k4_pass2_store_r8<10, 4>);
+  raise(k4_pass2_store_r8<11, 4>), raise(k4_pass2_store_r8<12, 2>);
+#define P2S(L) raise(k3_pass1<double2, L, FftCfg<double2>::kCols>), raise(k4_pass2_store<double2, L>),       \
               raise(k4_pass2_ip<double2, double, AccD, L, false>), raise(k4_pass2_ip<float2, float, AccF, L, false>), \
               raise(k4_pass2_ip<double2, double, AccD, L, true>), raise(k4_pass2_ip<float2, float, AccF, L, true>)
-  P2(5); P2(6); P2(7); P2(8); P2(9); P2(10); P2(11); P2(12);
-#undef P2
+  P2S(5); P2S(6); P2S(7);
+#undef P2S
+#define PX(L) raise(fxfft::k4_pass2_ip_fixed<L, false>), raise(fxfft::k4_pass2_ip_fixed<L, true>)
+  PX(8); PX(9); PX(10); PX(11); PX(12);
+#undef PX
+  raise(fxfft::k3_pass1_fixed<8, 8>), raise(fxfft::k3_pass1_fixed<9, 4>), raise(fxfft::k3_pass1_fixed<10, 2>);
+  raise(fxfft::k4_pass2_store_fixed<8, 2>), raise(fxfft::k4_pass2_store_fixed<9, 2>);
+  raise(fxfft::k4_pass2_store_fixed<10, 2>), raise(fxfft::k4_pass2_store_fixed<11, 2>);
+  raise(fxfft::k4_pass2_store_fixed<12, 1>);
 #define P3(L) raise(k4_pass2_ip_r8<L, false>), raise(k4_pass2_ip_r8<L, true>)
   P3(8); P3(9); P3(10); P3(11); P3(12);
 #undef P3

@@ -23,6 +23,7 @@
 // takes 0.04 ms for 8 and 0.05 ms for 1024.
 #include "emri_common.cuh"
 #include "emri_internal.h"
+#include "fx64.cuh"
 
 namespace emri {
 
@@ -268,7 +269,14 @@ __global__ void k0_delay_table(const WalkerC* __restrict__ wc, int n1, int n2, C
       vy = vx * ci + vy * cr;
       vx = t;
     }
-    *dst = make_double2(vx, vy);
+    // columns of 256 rows or more: the fixed-point pass 2 takes the factors as
+    // (cos.h, cos.l, sin.h, sin.l) in Q62
+    if (!row && n1 >= 256) {
+      const fx::Op a = fx::op(llrint(vx * 0x1p62)), b = fx::op(llrint(vy * 0x1p62));
+      *reinterpret_cast<int4*>(dst) = make_int4(a.h, a.l, b.h, b.l);
+    } else {
+      *dst = make_double2(vx, vy);
+    }
   }
 }
 
