@@ -248,7 +248,7 @@ struct OrbWork {
   double* start;   // [ns + 1][10]  compensated start states
   float* coarse;   // [ns / ratio][2][32] starting guess at the coarse nodes
   int* flag;       // [0] segments solved, [1] first segment with a bad knot, [2..4] sizes of the updates applied by
-                   // evaluations 1..3 (float bits), [5] segments the starting guess covers
+                   // evaluations 1..3 (float bits), [5] segments the starting guess covers, [6] first bad knot
 };
 constexpr int kOrbFlags = 8;
 
@@ -355,9 +355,7 @@ __global__ void __launch_bounds__(32) k1a_coarse(const WalkerC* __restrict__ wcs
         break;
       }
     }
-    // not settled, or past the LSO at some node: from here on in sequence
-    const bool past = !back && v * v >= (1.f - e * e) / (6.f + 2.f * e);
-    if (!conv || __any_sync(0xffffffffu, past)) {
+    if (!conv) {   // from here on in sequence
       good = g;
       break;
     }
@@ -370,8 +368,15 @@ __global__ void __launch_bounds__(32) k1a_coarse(const WalkerC* __restrict__ wcs
     fep = f0e;
     va = __shfl_sync(0xffffffffu, v, 31);
     ea = __shfl_sync(0xffffffffu, e, 31);
+    // past the LSO at some node: the last segment needed (the system is
+    // regular at the LSO)
+    if (__any_sync(0xffffffffu, !back && v * v >= (1.f - e * e) / (6.f + 2.f * e))) {
+      good = g + 1;
+      break;
+    }
   }
-  if (lane < kOrbFlags) o.flag[lane] = lane == 0 || lane == 5 ? good * ratio : lane == 1 ? (int)ns : 0;
+  if (lane < kOrbFlags)
+    o.flag[lane] = lane == 0 || lane == 5 ? good * ratio : lane == 1 ? (int)ns : lane == 6 ? (int)(n / ks) + 1 : 0;
 }
 
 // Correction (v, e) of segment i's start value, from the previous
@@ -706,7 +711,7 @@ __device__ __forceinline__ void knot_state(OrbState& y, const double* f5, const 
 // one segment, or in 32/K of them when a segment has K < 32 knots), and the
 // start knot.  ~400 FP64 instructions per knot, 160 of them the node sums:
 // bound by the FP64 pipe.  A knot past the LSO (forward) or not finite lowers
-// flag[1] to its segment.
+// flag[1] to its segment and flag[6] to itself.
 constexpr int kRateStride = 161;   // doubles per segment in shared memory (odd: no bank conflicts between segments)
 __global__ void __launch_bounds__(32) k1e_knots(const WalkerC* __restrict__ wcs, int64_t n, double dt,
                                                 const double2* __restrict__ cs, int ks, int pn, int back, int doppler,
@@ -740,6 +745,7 @@ __global__ void __launch_bounds__(32) k1e_knots(const WalkerC* __restrict__ wcs,
                (double)seg * dt * (back ? -1.0 : 1.0));
     if (!state_finite(y) || (!back && plunged(y.v_hi, y.e_hi))) {
       atomicMin(&o.flag[1], i);
+      atomicMin(&o.flag[6], (int)kq + 1);
     } else {
       const int64_t k = back ? nk - 1 - kq : kq + 1;
       ak_rhs_v(s, y.v_hi, y.e_hi, r[0], r[1], r[2], r[3], r[4]);
@@ -777,9 +783,54 @@ __device__ __forceinline__ OrbState bcast_state(const OrbState& a, int src) {
                   bcast(a.a_hi, src), bcast(a.a_lo, src)};
 }
 
+// One RK4 step of (v, e), rates (k1v, k1e) at the start.
+__device__ __forceinline__ void rk4_ve(const OrbSrc& s, double& v, double& e, double h, double k1v, double k1e) {
+  double k2v, k2e, k3v, k3e, k4v, k4e;
+  ak_rate_ve(s, v + 0.5 * h * k1v, e + 0.5 * h * k1e, k2v, k2e);
+  ak_rate_ve(s, v + 0.5 * h * k2v, e + 0.5 * h * k2e, k3v, k3e);
+  ak_rate_ve(s, v + h * k3v, e + h * k3e, k4v, k4e);
+  v += h / 6.0 * (k1v + 2.0 * (k2v + k3v) + k4v);
+  e += h / 6.0 * (k1e + 2.0 * (k2e + k3e) + k4e);
+}
+
+// Samples from a knot inside the LSO (state y0) to the first sample past it
+// (1..ks; the next knot is past it), by the whole warp: one RK4 step from the
+// knot to each 32nd of the interval, then one from the last of these inside
+// the LSO to each sample after it.  The steps are accurate where the state
+// moves slowly, which is checked: two half steps have to give the same
+// distance from the LSO to 1e-4 of what it changes by in one sample, else -1
+// (the caller steps through the samples).  ~1000 FP64 instructions in
+// sequence, 45 us; stepping sample by sample took ks times 12 us.
+__device__ int plunge_sample(const OrbSrc& s, const OrbState& y0, int ks, double dt, int lane) {
+  auto past = [](double v, double e) { return !(isfinite(v) && isfinite(e)) || plunged(v, e); };
+  auto margin = [](double v, double e) { return v * v * (6.0 + 2.0 * e) - (1.0 - e * e); };
+  const int sub = ks / 32;   // ks >= 64, a power of two
+  const double v0 = y0.v_hi + y0.v_lo, e0 = y0.e_hi + y0.e_lo, h = (double)((lane + 1) * sub) * dt;
+  double fv, fe;
+  ak_rate_ve(s, v0, e0, fv, fe);
+  double v = v0, e = e0, v2 = v0, e2 = e0, gv, ge;
+  rk4_ve(s, v, e, h, fv, fe);
+  rk4_ve(s, v2, e2, 0.5 * h, fv, fe);
+  ak_rate_ve(s, v2, e2, gv, ge);
+  rk4_ve(s, v2, e2, 0.5 * h, gv, ge);
+  const double rate = fabs(2.0 * v0 * (6.0 + 2.0 * e0) * fv + 2.0 * (v0 * v0 + e0) * fe) * dt;
+  if (!__all_sync(0xffffffffu, fabs(margin(v, e) - margin(v2, e2)) <= 1e-4 * rate)) return -1;
+  const unsigned b = __ballot_sync(0xffffffffu, past(v, e));
+  if (!b) return ks;
+  const int m = __ffs(b) - 1;                       // the crossing lies in (m sub, (m + 1) sub]
+  v = m ? bcast(v, m - 1) : v0;
+  e = m ? bcast(e, m - 1) : e0;
+  ak_rate_ve(s, v, e, fv, fe);
+  rk4_ve(s, v, e, (double)(lane + 1) * dt, fv, fe);
+  const unsigned c = __ballot_sync(0xffffffffu, lane < sub && past(v, e));
+  return m * sub + (c ? __ffs(c) : sub);
+}
+
 // The rest of a walker's orbit from its first segment that the parallel
 // solution does not cover (none for most walkers: then this only writes the
-// status), one warp per walker in sequence: per segment FP64 Picard sweeps,
+// status), one warp per walker.  A solved segment that passes the LSO at a
+// knot: the plunge sample (plunge_sample), the knots being there already.
+// Otherwise in sequence: per segment FP64 Picard sweeps,
 // the knots from the segment polynomial, and where the sweeps do not settle
 // or a knot lies past the LSO, knot-step RK4 by lane 0, which also locates the
 // plunge sample.  In backward mode no plunge check applies; an orbit that
@@ -804,9 +855,7 @@ __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_
   const uint32_t st0 = c.status;
   Knot* kn = knots + wk * (nk + 1);
   if (st0 & ST_BADPARAM) {
-    Knot zk = {};
-    for (int64_t k = lane; k <= nk; k += 32) kn[k] = zk;
-    if (lane == 0) wcs[wk].j_plunge = 0;
+    if (lane == 0) wcs[wk].j_plunge = 0;   // no sample and no knot is looked at
     return;
   }
   const OrbSrc s = orb_src(c, pn);
@@ -818,7 +867,27 @@ __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_
   bool fail = false;                // backward: the orbit turned non-finite
   const int64_t kstart = back ? nk - (int64_t)g0 * K : (int64_t)g0 * K;
   int64_t last = kstart;            // forward: last knot written
-  if (back && !state_finite(y)) {
+  bool done = false;
+  if (!back && g0 < o.flag[0]) {    // solved: the first knot past the LSO is q, counted from the segment's start
+    const int q = o.flag[6] - g0 * K;
+    const double* f5 = reinterpret_cast<const double*>(o.work + (int64_t)g0 * 1280);
+    OrbState ym = y, yq = y;        // knots q - 1 and q
+    if (q > 1) knot_state(ym, f5, qk_g + (size_t)(q - 1) * (128 / K) * 32, H);
+    knot_state(yq, f5, qk_g + (size_t)q * (128 / K) * 32, H);
+    const int d = state_finite(yq) ? plunge_sample(s, ym, ks, dt, lane) : -1;
+    if (d > 0) {
+      last = kstart + q;
+      jp = (last - 1) * ks + d;
+      if (jp < n) st |= ST_PLUNGE;
+      else jp = n;
+      double r[5];
+      ak_rhs_v(s, yq.v_hi, yq.e_hi, r[0], r[1], r[2], r[3], r[4]);
+      if (lane == 0) write_knot(kn, last, yq, r, c, cs, doppler);
+      done = true;
+    }
+  }
+  if (done) {
+  } else if (back && !state_finite(y)) {
     fail = true;
   } else {
     double r[5];
@@ -829,7 +898,7 @@ __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_
       st |= ST_PLUNGE;
     }
   }
-  for (int64_t g = g0; g < ns && jp == n && !fail; ++g) {
+  for (int64_t g = g0; g < ns && jp == n && !fail && !done; ++g) {
     const OrbState ys = y;          // segment start
     const int64_t kb = back ? nk - g * (int64_t)K : g * (int64_t)K;   // its knot
     double fv, fe;
@@ -910,9 +979,12 @@ __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_
     last = kb + K;
   }
   __syncwarp();
-  // forward: knots past a plunge repeat the last one written (their samples are zeroed)
+  // forward: knots past a plunge repeat the last one written, up to the end of
+  // the 4096 samples that the waveform kernels treat together (the samples
+  // after the plunge are zeroed, whole segments of them without the knots)
+  const int64_t kend = min(nk, last + 4096 / ks);
   if (!back)
-    for (int64_t q = last + 1 + lane; q <= nk; q += 32) kn[q] = kn[last];
+    for (int64_t q = last + 1 + lane; q <= kend; q += 32) kn[q] = kn[last];
   if (lane == 0) {
     wcs[wk].j_plunge = back ? (fail ? 0 : n) : jp;
     wcs[wk].status = st0 | st | (fail ? (uint32_t)ST_NONFINITE : 0u);

@@ -57,7 +57,7 @@ __device__ __forceinline__ T bessel_series(int m, T x, const T* __restrict__ bc,
   lead *= ifact[m];
   const T y = half * half;
   int K = (int)(T(12) + T(1.05) * x) + 1;
-  if (K > kBesselTerms) K = kBesselTerms;
+  if ((unsigned)(K - 1) >= (unsigned)kBesselTerms) K = kBesselTerms;
   const T* a = bc + m * kBesselTerms;
   T sum = a[K - 1];
 #pragma unroll 4
@@ -1068,6 +1068,10 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
   const int ni = ks >= kSegM ? 1 : kSegM / ks;
   const int t = threadIdx.x;
   const float scale = unit_scale ? C.gf.amp_scale : 1.f;
+  if (C.j_plunge <= j0) {   // nothing left of the inspiral
+    for (int r = t; r < kSegM; r += kTile) z[(int64_t)wk * n + j0 + r] = make_float2(0.f, 0.f);
+    return;
+  }
   if (t < ni) iv[t] = ivs[(int64_t)wk * nk + kfirst + t];
   if (t >= 128 && t < 128 + 4 * kTiles) {   // node q of tile tt
     const int i = t - 128, tt = i / 4, q = i % 4;
