@@ -14,9 +14,9 @@
 // (the same absolute size, on values that have grown by sqrt(8) per stage)
 // add less.  RMS error of a 2^20-point transform of noise: 2.4e-16 relative,
 // against 3.9e-16 in double.
-// 128 walkers x 2^21 (passes of 1024 and 2048 points): pass 1 17.6 -> 5.7 ms,
-// pass 2 with the inner products 23.2 -> 6.8 ms; 23 transforms of 2^19 points
-// 1.49 -> 0.51 ms.
+// 128 walkers x 2^21 (passes of 1024 and 2048 points): pass 1 17.6 -> 3.7 ms,
+// pass 2 with the inner products 23.2 -> 4.2 ms; 23 transforms of 2^19 points
+// 1.49 -> 0.38 ms.
 // Transforms that hold NaN, infinities, or numbers outside [1e-30, 1e30] in
 // sum take the FP64 Stockham form (their CTA does).
 #pragma once
@@ -153,6 +153,16 @@ __device__ __forceinline__ double from_fixed(i64 v, int k) {
   return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) - (k << 20), __double2loint(d));
 }
 
+// v 2^-k for v = 0 or 2^32 <= v < 2^63, on the integer pipe (a conversion
+// takes the FP64 pipe for 64 cycles): round to 53 bits, the leading bit carries
+// into the exponent
+__device__ __forceinline__ double from_fixed_pos(i64 v, int k) {
+  const int lz = __clz(fx::hi(v));
+  const fx::u64 m = (((fx::u64)v << (lz - 1)) + 0x200) >> 10;
+  const double d = __longlong_as_double((long long)(m + ((fx::u64)(1085 - lz - k) << 52)));
+  return v == 0 ? 0.0 : d;
+}
+
 template <int LG, int NB>
 struct Cfg {
   static constexpr int N = 1 << LG, T = N / 8, kThreads = NB * T;
@@ -278,11 +288,11 @@ __device__ __forceinline__ double2 out2(Z v, int k, bool swap) {
 
 // Pass 1: NB adjacent columns j1, with the inter-pass twiddle W_n^{j1 k2} on
 // the way out: W^{j1 t} of the thread times W^{j1 T q}, one per column and slot.
-// 256 threads a CTA (NB = 2, 4, 8 columns of 1024, 512, 256 points), two CTAs
-// per SM at 128 registers: one CTA's loads and stores run beside the other's
+// 256 threads a CTA (NB = 2, 4, 8 columns of 1024, 512, 256 points), three CTAs
+// per SM at 80 registers: one CTA's loads and stores run beside the others'
 // stages.
 template <int LG, int NB>
-__global__ void __launch_bounds__(Cfg<LG, NB>::kThreads, 2)
+__global__ void __launch_bounds__(Cfg<LG, NB>::kThreads, 3)
     k3_pass1_fixed(const double2* zin, double2* zout, int64_t n, int n1, int sign, int shift22, const double2* __restrict__ ta,
                    const double2* __restrict__ tb, const double2* __restrict__ tc) {
   using F = Cfg<LG, NB>;
@@ -352,7 +362,7 @@ __global__ void __launch_bounds__(Cfg<LG, NB>::kThreads, Cfg<LG, NB>::kThreads >
 // conversions and five FP64 FMAs per bin remain (twelve in double), and run
 // beside the integer work.
 template <int LG, bool FD>
-__global__ void __launch_bounds__(Cfg<LG, 1>::kThreads, Cfg<LG, 1>::kThreads > 256 ? 1 : 512 / Cfg<LG, 1>::kThreads)
+__global__ void __launch_bounds__(Cfg<LG, 1>::kThreads, Cfg<LG, 1>::kThreads > 256 ? 1 : 768 / Cfg<LG, 1>::kThreads)
     k4_pass2_ip_fixed(const double2* __restrict__ y, int64_t n, int n2, const double2* __restrict__ tc,
                       const WalkerC* __restrict__ wcs, const int4* __restrict__ dtab, const double2* __restrict__ rtab,
                       const double2* __restrict__ dperm, const double* __restrict__ wperm,
@@ -391,9 +401,9 @@ __global__ void __launch_bounds__(Cfg<LG, 1>::kThreads, Cfg<LG, 1>::kThreads > 2
       double2 P = make_double2(from_fixed(Pi.x, sh), from_fixed(Pi.y, sh));
       // the one negative bin of this column not in the table: k1 = N/2 = 4 T
       if (q == 4 && t == 0 && k2 > 0) P = ::emri::cmul(P, cnv);
-      zr += G.x * P.x - G.y * P.y;
-      zi += G.x * P.y + G.y * P.x;
-      shh += wv * from_fixed(h2.get(), 2 * sh);
+      zr = fma(-G.y, P.y, fma(G.x, P.x, zr));
+      zi = fma(G.y, P.x, fma(G.x, P.y, zi));
+      shh = fma(wv, from_fixed_pos(h2.get(), 2 * sh), shh);
     }
   } else {
     FdW fd;
@@ -420,8 +430,8 @@ __global__ void __launch_bounds__(Cfg<LG, 1>::kThreads, Cfg<LG, 1>::kThreads > 2
         P = ::emri::cmul(P, make_double2(A * cf, A * sf));
         A2 = A * A;
       }
-      zr += G.x * P.x - G.y * P.y;
-      zi += G.x * P.y + G.y * P.x;
+      zr = fma(-G.y, P.y, fma(G.x, P.x, zr));
+      zi = fma(G.y, P.x, fma(G.x, P.y, zi));
       shh += __ldg(ws + k1) * (H.x * H.x + H.y * H.y) * A2;
     }
   }
