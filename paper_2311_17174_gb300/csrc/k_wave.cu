@@ -126,6 +126,8 @@ __device__ double2 g_exp512[kExpLen];
 // exp(2 pi i k / 1024) in Q62 for the fixed-point sin/cos
 __device__ fx::Trig g_trig[fx::kTrigLen];
 
+static bool wave_smem_limits();
+
 int upload_exp512() {
   double2 h[kExpLen];
   const long double pi = 3.141592653589793238462643383279502884L;
@@ -139,7 +141,7 @@ int upload_exp512() {
     q[k].c = llrintl(cosl(a) * 0x1p62L);
     q[k].s = llrintl(sinl(a) * 0x1p62L);
   }
-  const bool ok = cudaMemcpyToSymbol(g_exp512, h, sizeof(h)) == cudaSuccess &&
+  const bool ok = wave_smem_limits() && cudaMemcpyToSymbol(g_exp512, h, sizeof(h)) == cudaSuccess &&
                   cudaMemcpyToSymbol(g_trig, q.data(), q.size() * sizeof(fx::Trig)) == cudaSuccess;
   return ok ? 0 : -1;
 }
@@ -292,17 +294,6 @@ void launch_lisa(int64_t n, int ks, double t0, double dt, double* tab, cudaStrea
   k_lisa<<<(unsigned)((4 * nt + nkn + 127) / 128), 128, 0, s>>>(nt, nkn, ks, t0, dt, tab);
 }
 
-// fixed-point phase: (base + tau*inc) mod 1 to 32 bits, plus the FP32
-// correction c2 s^2 + c3 s^3; returns the phase in cycles in [-0.5, 0.5)
-__device__ __forceinline__ float phase_fx(unsigned long long base, long long inc, const float c[2], int tau,
-                                          float s) {
-  const unsigned long long p = base + (unsigned long long)tau * (unsigned long long)inc;   // mod 2^64
-  const int top = (int)(unsigned)(p >> 32);
-  float f = (float)top * 2.3283064365386963e-10f;  // 2^-32
-  f += (c[1] * s + c[0]) * s * s;
-  return f - rintf(f);
-}
-
 // --------------------------------------------------- response + harmonics
 template <typename T>
 __device__ __forceinline__ T rcp_fast(T x) { return T(1) / x; }
@@ -369,11 +360,6 @@ __device__ __forceinline__ void harmonic_sums(double cph, double sph, double st,
     hs.next();
   }
 }
-
-// FP32 amplitude coefficients per harmonic, each stored twice so that the
-// paired (f32x2) instructions of harmonic_sums4 take natural register pairs:
-// (a0 a0 a1 a1)(a2 a2 b0 b0)(b1 b1 b2 b2)(r0 r0 r1 r1)(r2 r2 - -).
-constexpr int kAmpStrideM = 20;
 
 // ----------------------------------------------------------- response
 // The LISA response of Sec. 2 (Eq. 2 with the Barack-Cutler antenna
@@ -491,31 +477,53 @@ __device__ __forceinline__ void channels(const Geo<double>& g, double cph, doubl
 }
 
 
+// quadratic in [0, 1] through f0, fh, f1 at 0, 1/2, 1
+template <typename T>
+__device__ __forceinline__ void fit3(T f0, T fh, T f1, T* q) {
+  q[0] = f0;
+  q[1] = T(-3) * f0 + T(4) * fh - f1;
+  q[2] = T(2) * f0 - T(4) * fh + T(2) * f1;
+}
+
+// Amplitudes of one harmonic over a block of kBlk samples: a, b, c as
+// A0 + A1 u + A2 u^2 in the sample offset u from the block's centre, each
+// coefficient twice, so that the paired (f32x2) instructions of harmonic_sums4
+// take natural register pairs.
+struct __align__(16) BlkAmp {
+  float4 a, b, c;   // (A0, A0, A1, A1)
+  float4 ab2, c2;   // (A2 of a, twice, A2 of b, twice), (A2 of c, twice, -, -)
+};
+constexpr int kBlk = 128;
+
 // FP32, four samples at once, as two (A, B) pairs of every quantity --
 // cos(n Phi), sin(n Phi), the three amplitudes and the three sums -- so each
 // step is one paired (f32x2) instruction on operands that are natural
-// register pairs, and the coefficients of a harmonic (five 16-byte loads) are
-// loaded once for all four samples.  c1, s1: cos, sin of the Doppler orbital
-// phase; st: fit times in [0, 1]; C, S, R: sum_n a_n cos(n Phi),
-// sum_n b_n sin(n Phi), sum_n c_n cos(n Phi).
-__device__ __forceinline__ void harmonic_sums4(const float2 (&c1)[2], const float2 (&s1)[2], const float2 (&st)[2],
-                                               const float* __restrict__ bq, int n_max, bool cheb, float2 (&C)[2],
+// register pairs, and the coefficients of a harmonic (three 16-byte loads, five
+// with kCurved) are loaded once for all four samples.  c1, s1: cos, sin of the
+// Doppler orbital phase; u: offsets from the block's centre; C, S, R: sum_n a_n
+// cos(n Phi), sum_n b_n sin(n Phi), sum_n c_n cos(n Phi).
+template <bool kCurved>
+__device__ __forceinline__ void harmonic_sums4(const float2 (&c1)[2], const float2 (&s1)[2], const float2 (&u)[2],
+                                               const BlkAmp* __restrict__ amp, int n_max, bool cheb, float2 (&C)[2],
                                                float2 (&S)[2], float2 (&R)[2]) {
   for (int p = 0; p < 2; ++p) C[p] = S[p] = R[p] = make_float2(0.f, 0.f);
   auto harm = [&](int n, const float2 (&c)[2], const float2 (&sn)[2]) {
-    const float4* b = reinterpret_cast<const float4*>(bq + kAmpStrideM * n);
-    const float4 x0 = b[0], x1 = b[1], x2 = b[2], x3 = b[3], x4 = b[4];
+    const float4 xa = amp[n].a, xb = amp[n].b, xc = amp[n].c;
+    float2 a1[2] = {hi2(xa), hi2(xa)}, b1[2] = {hi2(xb), hi2(xb)}, r1[2] = {hi2(xc), hi2(xc)};
+    if (kCurved) {
+      const float4 y = amp[n].ab2, w = amp[n].c2;
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        a1[p] = __ffma2_rn(lo2(y), u[p], a1[p]);
+        b1[p] = __ffma2_rn(hi2(y), u[p], b1[p]);
+        r1[p] = __ffma2_rn(lo2(w), u[p], r1[p]);
+      }
+    }
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-      const float2 a = __ffma2_rn(__ffma2_rn(make_float2(x1.x, x1.y), st[p], make_float2(x0.z, x0.w)), st[p],
-                                  make_float2(x0.x, x0.y));
-      const float2 bb = __ffma2_rn(__ffma2_rn(make_float2(x2.z, x2.w), st[p], make_float2(x2.x, x2.y)), st[p],
-                                   make_float2(x1.z, x1.w));
-      const float2 r = __ffma2_rn(__ffma2_rn(make_float2(x4.x, x4.y), st[p], make_float2(x3.z, x3.w)), st[p],
-                                  make_float2(x3.x, x3.y));
-      C[p] = __ffma2_rn(a, c[p], C[p]);
-      S[p] = __ffma2_rn(bb, sn[p], S[p]);
-      R[p] = __ffma2_rn(r, c[p], R[p]);
+      C[p] = __ffma2_rn(__ffma2_rn(a1[p], u[p], lo2(xa)), c[p], C[p]);
+      S[p] = __ffma2_rn(__ffma2_rn(b1[p], u[p], lo2(xb)), sn[p], S[p]);
+      R[p] = __ffma2_rn(__ffma2_rn(r1[p], u[p], lo2(xc)), c[p], R[p]);
     }
   };
   float2 cu[2] = {c1[0], c1[1]}, su[2] = {s1[0], s1[1]};
@@ -527,18 +535,18 @@ __device__ __forceinline__ void harmonic_sums4(const float2 (&c1)[2], const floa
       harm(n, cu, su);
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
-        cv[p] = __ffma2_rn(tc[p], cu[p], make_float2(-cv[p].x, -cv[p].y));
-        sv[p] = __ffma2_rn(tc[p], su[p], make_float2(-sv[p].x, -sv[p].y));
+        cv[p] = __ffma2_rn(tc[p], cu[p], neg2(cv[p]));
+        sv[p] = __ffma2_rn(tc[p], su[p], neg2(sv[p]));
       }
       harm(n + 1, cv, sv);
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
-        cu[p] = __ffma2_rn(tc[p], cv[p], make_float2(-cu[p].x, -cu[p].y));
-        su[p] = __ffma2_rn(tc[p], sv[p], make_float2(-su[p].x, -su[p].y));
+        cu[p] = __ffma2_rn(tc[p], cv[p], neg2(cu[p]));
+        su[p] = __ffma2_rn(tc[p], sv[p], neg2(su[p]));
       }
     }
   } else {
-    const float2 ns[2] = {make_float2(-s1[0].x, -s1[0].y), make_float2(-s1[1].x, -s1[1].y)};
+    const float2 ns[2] = {neg2(s1[0]), neg2(s1[1])};
     for (; n + 1 < n_max; n += 2) {
       harm(n, cu, su);
       float2 cv[2], sv[2];
@@ -558,65 +566,36 @@ __device__ __forceinline__ void harmonic_sums4(const float2 (&c1)[2], const floa
   if (n < n_max) harm(n, cu, su);
 }
 
-// Per-harmonic amplitude coefficients in shared memory: 9 values (a, b, c
-// quadratics) at stride AmpStride<T>; FP32 stores each twice in the layout
-// of harmonic_sums4 (five 16-byte loads per harmonic).
-template <typename T>
-struct AmpStride;
-template <>
-struct AmpStride<double> {
-  static constexpr int v = 9;
-};
-template <>
-struct AmpStride<float> {
-  static constexpr int v = kAmpStrideM;
-};
+// Bessel amplitudes of a segment (FP32): nodes at sample offsets 0, L/2, L
+// (L = span: the segment's length, or the last valid offset when the orbit
+// plunges inside it), fitted by quadratics in t / L: bq[n][3 f + p] =
+// coefficient p of quantity f.
+constexpr int kQuadStride = 12;
 
-// Bessel amplitude fit for the tile: nodes at tile-relative sample offsets
-// 0, L/2, L (L = 256, or the last valid offset when the orbit plunges inside
-// the tile), quadratic in st = t / L.
-template <typename T, typename IV>
-__device__ __forceinline__ void tile_harmonics(const IV* iv, int ni, int64_t j0, int64_t kfirst, int ks,
-                                               int n_max, int span, T* bnode, T* bq, const T* __restrict__ bc,
-                                               const T* __restrict__ ifact) {
+__device__ __forceinline__ void tile_harmonics(const IvM* iv, int ni, int64_t j0, int64_t kfirst, int ks, int n_max,
+                                               int span, float* bnode, float* bq, const float* __restrict__ bc,
+                                               const float* __restrict__ ifact) {
   const int t = threadIdx.x;
   if (t < 3 * n_max) {
     // harmonic-major: a warp holds neighbouring n, whose series lengths
     // (growing with x = n e) are alike
     const int node = t % 3, n = t / 3 + 1;
     // node at offset span*node/2: integer arithmetic in half samples, so no
-    // FP64 instruction runs here in the FP32 kernel
+    // FP64 instruction runs here
     const int64_t pos2 = 2 * j0 + (int64_t)span * node;
     int64_t ki = pos2 / (2 * ks) - kfirst;
     if (ki > ni - 1) ki = ni - 1;
     if (ki < 0) ki = 0;
     const int64_t rem2 = pos2 - 2 * (kfirst + ki) * ks;
-    const T s = T(rem2) / T(2 * ks);
-    const T e = T(iv_e(iv[ki], s));
-    T out[3];
-    harmonic_amps<T>(n, e, out, bc, ifact);
-    bnode[(node * 32 + (n - 1)) * 3 + 0] = out[0];
-    bnode[(node * 32 + (n - 1)) * 3 + 1] = out[1];
-    bnode[(node * 32 + (n - 1)) * 3 + 2] = out[2];
+    float out[3];
+    harmonic_amps<float>(n, iv_e(iv[ki], (float)rem2 / (float)(2 * ks)), out, bc, ifact);
+    for (int f = 0; f < 3; ++f) bnode[(node * 32 + (n - 1)) * 3 + f] = out[f];
   }
   __syncthreads();
   if (t < 3 * n_max) {
     const int n = t / 3, f = t % 3;
-    const T f0 = bnode[(0 * 32 + n) * 3 + f], fh = bnode[(1 * 32 + n) * 3 + f], f1 = bnode[(2 * 32 + n) * 3 + f];
-    const T q0 = f0, q1 = T(-3) * f0 + T(4) * fh - f1, q2 = T(2) * f0 - T(4) * fh + T(2) * f1;
-    T* o = bq + AmpStride<T>::v * n;
-    if (sizeof(T) == 4) {                // FP32: quantity f, coefficient p at 6 f + 2 p and the next
-      o[6 * f + 0] = q0;
-      o[6 * f + 1] = q0;
-      o[6 * f + 2] = q1;
-      o[6 * f + 3] = q1;
-      o[6 * f + 4] = q2;
-      o[6 * f + 5] = q2;
-    } else {
-      o[3 * f + 0] = q0;
-      o[3 * f + 1] = q1;
-      o[3 * f + 2] = q2;
-    }
+    fit3(bnode[(0 * 32 + n) * 3 + f], bnode[(1 * 32 + n) * 3 + f], bnode[(2 * 32 + n) * 3 + f],
+         bq + kQuadStride * n + 3 * f);
   }
 }
 
@@ -629,13 +608,6 @@ __device__ __forceinline__ int tile_span(int64_t j0, int64_t jp, int L = kTile) 
 }
 
 // ------------------------------------------------------------- kernels
-template <typename T>
-__device__ __forceinline__ void fit3(T f0, T fh, T f1, T* q) {
-  q[0] = f0;
-  q[1] = T(-3) * f0 + T(4) * fh - f1;
-  q[2] = T(2) * f0 - T(4) * fh + T(2) * f1;
-}
-
 // Above these sample intervals the per-tile cubic of the antenna patterns
 // (error ~ (256 dt / T)^4) is replaced by their exact value per sample.
 constexpr double kPatternFitDtMax64 = 64.0;     // [s]; fit error < 2e-12 below
@@ -649,7 +621,7 @@ constexpr double kPatternFitDtMaxM = 1024.0;    // [s]; fit error < 1e-7 below
 constexpr int kSegF = 1024;
 
 // The samples of a segment in double, for the segments the fixed-point form
-// does not take (wave_fixed_ok): long sample intervals, whose antenna patterns
+// does not take: long sample intervals, whose antenna patterns
 // are exact per sample, and orbits or geometries outside its ranges.
 __device__ __noinline__ void wave_samples_f64(const IvD* iv, const double* bq, const double (*fq)[4][4],
                                               const Geo<double>& g, int64_t j0, int64_t kfirst, int64_t jplunge,
@@ -666,7 +638,7 @@ __device__ __noinline__ void wave_samples_f64(const IvD* iv, const double* bq, c
     const int64_t j = j0 + r;
     double2 out = make_double2(0.0, 0.0);
     if (j < jplunge) {
-      const int ki = ks >= kSegF ? 0 : r >> lks;
+      const int ki = (int)((j >> lks) - kfirst);
       const double s = (double)(j - (kfirst + ki) * ks) * (1.0 / (double)ks);
       const IvD& v = iv[ki];
       // phases in cycles over the knot interval (|f| < 2^20: the table index
@@ -773,7 +745,7 @@ __device__ __forceinline__ double pow2d(int k) { return __longlong_as_double((lo
 // double.  Per harmonic 8 multiply-adds advance cosine and sine, 9 add the
 // constant, 9 the linear and 3 the quadratic coefficients (which are ~2^-9 and
 // ~2^-20 of the constant ones, so q2 mostly keeps one word, else kTwo): 29
-// multiply-adds and 8 others, ~145 cycles a warp, for 11 FP64 instructions
+// multiply-adds and ~12 others, ~150 cycles a warp, for 11 FP64 instructions
 // (836 cycles).
 template <bool kTwo>
 FX_HD void harmonics_fixed(fx::Trig cs, int r, const HarmX* __restrict__ hx, int n_max, int sh1,
@@ -877,148 +849,188 @@ FX_HD void response_fixed(const GeoX& g, fx::Trig gm, fx::Trig al, fx::i64 Cs, f
   Hx = u.get() + w.get();
 }
 
-// What bounds it: FP64 issue (1 warp instruction per 76 cycles).  In double a
-// sample takes 333 FP64 instructions at n_max = 20: 156.3 ms for 128 walkers x
-// 2^21 samples, 6.73 ms for 8 walkers x 2^21 at n_max = 10.  Here the phases,
-// their sines and cosines, the harmonic sums and the response run in 64-bit
-// fixed point on the integer pipe (~4200 cycles a warp at n_max = 20), and
-// only the slowly varying factors (x^(2/3), the patterns) stay in double,
-// beside them: 24 FP64 instructions.  56.7 and 2.59 ms.
-__global__ void __launch_bounds__(kTile, 2) k2_wave_f64(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
+// Shared memory of one FP64 waveform CTA (kSub segments of kSegF samples).
+template <int kSub>
+struct WaveSmem {
+  IvD iv[kSub * kSegF / 64];
+  IvX ivx[kSub * kSegF / 64];
+  fx::Trig ex[fx::kTrigLen];
+  HarmX hx[kSub][32];
+  double bnode[kSub][32][3][3];                // amplitudes [harmonic][a, b, c][node]
+  double bq[kSub][32 * 9];
+  double fn[kSub * kSegF / kTile][4][4];       // the four patterns at the four fit nodes of each tile
+  double fq[kSub * kSegF / kTile][4][4];       // their cubics in (t mod 256) / 256
+  Geo<double> g;
+  GeoX gx;
+  HarmScale hsc[kSub];
+  int fixed_bad[kSub];
+};
+
+// In double a sample takes 333 FP64 instructions at n_max = 20, 76 cycles each:
+// 156.3 ms for 128 walkers x 2^21 samples, 6.73 ms for 8 walkers x 2^21 at
+// n_max = 10.  Here the phases, their sines and cosines, the harmonic sums and
+// the response run in 64-bit fixed point on the integer pipe, ~800
+// multiply-adds of 4 cycles and ~900 other instructions a sample at n_max = 20,
+// and only the slowly varying factors (x^(2/3), the patterns) stay in double,
+// beside them: 24 FP64 instructions.  30.1 and 1.35 ms, bound by the
+// multiply-adds (~4500 cycles a warp in all).
+//
+// One CTA takes kSub segments: the set-up (Bessel amplitudes at three nodes a
+// segment, antenna patterns, interval records) is a serial chain of ~200 FP64
+// instructions, 20000 cycles, that few threads have work for in a single
+// segment; four segments fill the CTA's warps with it and pay its latency once
+// (56.7 -> 49.2 ms when the sums were slower).  A segment's result does not
+// depend on kSub.  Three CTAs per SM at 80 registers: 30.8 -> 30.1 ms against
+// two at 126, 16 sources x 2^16 0.141 -> 0.128 ms.
+template <int kSub>
+__global__ void __launch_bounds__(kTile, 3) k2_wave_f64(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
                                                         int64_t n, double dt, double t0, int ks, int n_max,
                                                         double2* __restrict__ z, int unit_scale, int exact_f,
                                                         const double* __restrict__ bc, const double* __restrict__ ifact,
                                                         const double* __restrict__ lisa) {
-  constexpr int kTiles = kSegF / kTile;
-  __shared__ IvD iv[kSegF / 64];
-  __shared__ IvX ivx[kSegF / 64];
-  __shared__ double bnode[3 * 32 * 3];
-  __shared__ double bq[32 * 9];
-  __shared__ HarmX hx[32];
-  __shared__ HarmScale hsc;
-  __shared__ double fn[kTiles][4][4];   // the four patterns at the four fit nodes of each tile
-  __shared__ double fq[kTiles][4][4];   // their cubics in (t mod 256) / 256
-  __shared__ fx::Trig ex[fx::kTrigLen];
-  __shared__ Geo<double> g;
-  __shared__ GeoX gx;
-  __shared__ int fixed_bad;
+  constexpr int kSub4 = kSegF / kTile, kTiles = kSub * kSub4;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  WaveSmem<kSub>& S = *reinterpret_cast<WaveSmem<kSub>*>(smraw);
   const int wk = blockIdx.y;
   const WalkerC& C = wcs[wk];
   const int64_t nk = n / ks;
   const Knot* kn = knots + (int64_t)wk * (nk + 1);
-  const int64_t j0 = (int64_t)blockIdx.x * kSegF;
-  const int64_t kfirst = j0 / ks;
-  const int ni = ks >= kSegF ? 1 : kSegF / ks;
+  const int64_t j0 = (int64_t)blockIdx.x * (kSub * kSegF);
+  const int lks = __ffs(ks) - 1;   // ks: a power of two, at most kSegF
+  const int64_t kfirst = j0 >> lks;
+  const int nis = kSegF >> lks;    // knot intervals per segment
   const int t = threadIdx.x;
   const double h = (double)ks * dt;
   const double scale = unit_scale ? C.gd.amp_scale : 1.0;
   z += (int64_t)wk * n;
   const int64_t jplunge = C.j_plunge;
   if (jplunge <= j0) {   // nothing left of the inspiral
-    for (int r = t; r < kSegF; r += kTile) z[j0 + r] = make_double2(0.0, 0.0);
+    for (int r = t; r < kSub * kSegF; r += kTile) z[j0 + r] = make_double2(0.0, 0.0);
     return;
   }
-  if (t == 0) fixed_bad = exact_f;
+  if (t < kSub) S.fixed_bad[t] = exact_f;
   __syncthreads();
-  if (t < ni) {
-    build_iv(kn[kfirst + t], kn[kfirst + t + 1], h, iv[t]);
-    const bool ok0 = phase_fixed(iv[t].ph, ks, ivx[t].ph), ok1 = phase_fixed(iv[t].gm, ks, ivx[t].gm),
-               ok2 = phase_fixed(iv[t].al, ks, ivx[t].al);
-    if (!(ok0 && ok1 && ok2)) fixed_bad = 1;
+  if (t < kSub * nis) {
+    build_iv(kn[kfirst + t], kn[kfirst + t + 1], h, S.iv[t]);
+    const bool ok0 = phase_fixed(S.iv[t].ph, ks, S.ivx[t].ph), ok1 = phase_fixed(S.iv[t].gm, ks, S.ivx[t].gm),
+               ok2 = phase_fixed(S.iv[t].al, ks, S.ivx[t].al);
+    if (!(ok0 && ok1 && ok2)) S.fixed_bad[t / nis] = 1;
   }
-  if (t >= 224 && t < 224 + 4 * kTiles && !exact_f) {   // node q of tile tt
-    const int i = t - 224, tt = i / 4, q = i % 4;
+  if (t >= 256 - 4 * kTiles && !exact_f) {   // node q of tile tt
+    const int i = t - (256 - 4 * kTiles), tt = i / 4, q = i % 4;
     const double* L = lisa + ((int64_t)blockIdx.x * kTiles + tt) * 8 + 2 * q;
-    antenna_fixed<double>(C.gd, L[0], L[1], scale, fn[tt][q]);
+    antenna_fixed<double>(C.gd, L[0], L[1], scale, S.fn[tt][q]);
   }
   if (t >= 160 && t < 170) {   // geometry constants, one per thread
     const Geo<double>& G = C.gd;
     const int i = t - 160;
     const double v = i == 0 ? G.pe1 : i == 1 ? -G.pe2 : i == 2 ? G.qe1 : i == 3 ? -G.qe2 : i == 4 ? G.cpe1
                    : i == 5 ? G.cpe2 : i == 6 ? G.cqe1 : i == 7 ? G.cqe2 : i == 8 ? -G.spS : -G.sqS;
-    if (!(fabs(v) < 1.0000001)) fixed_bad = 1;
-    if (i < 8) (&gx.pe1)[i] = fx::op(llrint(v * 0x1p62));
-    else (&gx.spSn)[i - 8] = llrint(v * 0x1p60);
-    if (i == 0) g = G;
+    if (!(fabs(v) < 1.0000001))
+      for (int q = 0; q < kSub; ++q) S.fixed_bad[q] = 1;
+    if (i < 8) (&S.gx.pe1)[i] = fx::op(llrint(v * 0x1p62));
+    else (&S.gx.spSn)[i - 8] = llrint(v * 0x1p60);
+    if (i == 0) S.g = G;
   }
-  for (int i = t; i < fx::kTrigLen; i += kTile) ex[i] = g_trig[i];
+  for (int i = t; i < fx::kTrigLen; i += kTile) S.ex[i] = g_trig[i];
   __syncthreads();
-  const int span = tile_span(j0, jplunge, kSegF);
-  tile_harmonics<double, IvD>(iv, ni, j0, kfirst, ks, n_max, span, bnode, bq, bc, ifact);
+  // Bessel amplitudes at a segment's start, middle and end (or last sample
+  // before a plunge); neighbouring threads hold the same harmonic, whose
+  // series lengths are alike
+  for (int i = t; i < 3 * kSub * n_max; i += kTile) {
+    const int m = i / (3 * kSub), sub = i % (3 * kSub) / 3, node = i % 3;
+    const int64_t js = j0 + sub * kSegF;
+    const int span = tile_span(js, jplunge, kSegF);
+    const int64_t pos2 = 2 * js + (int64_t)span * node;   // in half samples
+    int ki = (int)((pos2 >> (lks + 1)) - kfirst);
+    if (ki > (sub + 1) * nis - 1) ki = (sub + 1) * nis - 1;
+    const double s = (double)(pos2 - 2 * (kfirst + ki) * ks) / (double)(2 * ks);
+    double out[3];
+    harmonic_amps<double>(m + 1, iv_e(S.iv[ki], s), out, bc, ifact);
+    for (int f = 0; f < 3; ++f) S.bnode[sub][m][f][node] = out[f];
+  }
   __syncthreads();
-  if (t < 32) {   // block exponents
-    const float rs = (float)kSegF / (float)span;
+  if (t < 32 * kSub) {   // quadratics and block exponents, a warp per segment and a lane per harmonic
+    const int sub = t >> 5, m = t & 31;
+    const float rs = (float)kSegF / (float)tile_span(j0 + sub * kSegF, jplunge, kSegF);
     float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-    if (t < n_max)
+    if (m < n_max)
       for (int f = 0; f < 3; ++f) {
-        const double* b = bq + 9 * t + 3 * f;
-        s0 += fabsf((float)b[0]);
-        s1 += fabsf((float)b[1]) * rs;
-        s2 += fabsf((float)b[2]) * (rs * rs);
+        const double* b = S.bnode[sub][m][f];
+        double* o = S.bq[sub] + 9 * m + 3 * f;
+        fit3(b[0], b[1], b[2], o);
+        s0 += fabsf((float)o[0]);
+        s1 += fabsf((float)o[1]) * rs;
+        s2 += fabsf((float)o[2]) * (rs * rs);
       }
     for (int off = 16; off > 0; off >>= 1) {
       s0 += __shfl_xor_sync(0xffffffffu, s0, off);
       s1 += __shfl_xor_sync(0xffffffffu, s1, off);
       s2 += __shfl_xor_sync(0xffffffffu, s2, off);
     }
-    if (t == 0) {
-      hsc = harm_scale(1.0001f * s0, 1.0001f * s1, 1.0001f * s2);
+    if (m == 0) {
+      S.hsc[sub] = harm_scale(1.0001f * s0, 1.0001f * s1, 1.0001f * s2);
       // amplitudes that move by more than 1/32 of their sum over the segment
       // (the unit of q0 follows 128 S1) or are not finite: in double
-      if (!(s0 < 1e12f && 32.f * s1 < s0 && s2 < s0)) fixed_bad = 1;
+      if (!(s0 < 1e12f && 32.f * s1 < s0 && s2 < s0)) S.fixed_bad[sub] = 1;
     }
   }
   __syncthreads();
-  const bool fixed = !fixed_bad;
-  if (fixed) {
-    const double rs = (double)kSegF / (double)span;
-    for (int i = t; i < 9 * n_max; i += kTile) {
-      const int m = i / 9, f = (i % 9) / 3, p = i % 3;
-      double v = bq[i];
-      if ((m + 1) & 2) v = -v;   // the signs of the recurrence
-      v *= p == 0 ? pow2d(hsc.k0) : p == 1 ? pow2d(hsc.k1) * rs : pow2d(hsc.k2) * (rs * rs);
-      const fx::i64 q = llrint(v);
-      int* o = reinterpret_cast<int*>(hx + m);
-      int* oh = p < 2 ? o + 4 * f + 2 * p : hx[m].h2 + f;
-      int* ol = p < 2 ? oh + 1 : hx[m].l2 + f;
-      const bool one = p == 2 && !hsc.two;
-      *oh = (int)(one ? q : q >> 27);
-      *ol = one ? 0 : (int)(q & ((1 << 27) - 1));
+  for (int i = t; i < 9 * kSub * n_max; i += kTile) {
+    const int sub = i / (9 * n_max), r = i % (9 * n_max), m = r / 9, f = (r % 9) / 3, p = r % 3;
+    const HarmScale hs = S.hsc[sub];
+    const int span = tile_span(j0 + sub * kSegF, jplunge, kSegF);
+    double v = S.bq[sub][r];
+    if ((m + 1) & 2) v = -v;   // the signs of the recurrence
+    v *= pow2d(p == 0 ? hs.k0 : p == 1 ? hs.k1 : hs.k2);
+    if (span != kSegF) {       // the fit's time to rho = r / 1024
+      const double rs = (double)kSegF / (double)span;
+      v *= p == 0 ? 1.0 : p == 1 ? rs : rs * rs;
     }
+    const fx::i64 q = llrint(v);
+    HarmX& o = S.hx[sub][m];
+    int* oh = p < 2 ? reinterpret_cast<int*>(&o) + 4 * f + 2 * p : o.h2 + f;
+    int* ol = p < 2 ? oh + 1 : o.l2 + f;
+    const bool one = p == 2 && !hs.two;
+    *oh = (int)(one ? q : q >> 27);
+    *ol = one ? 0 : (int)(q & ((1 << 27) - 1));
   }
-  if (t >= 224 && t < 224 + 4 * kTiles && !exact_f) {   // pattern q of tile tt, in the sums' unit
-    const int i = t - 224, tt = i / 4, q = i % 4;
-    const double u = fixed ? pow2d(-2 - hsc.k0) : 1.0;
-    fit_cubic4<double>(u * fn[tt][0][q], u * fn[tt][1][q], u * fn[tt][2][q], u * fn[tt][3][q], fq[tt][q]);
+  if (t >= 256 - 4 * kTiles && !exact_f) {   // pattern q of tile tt, in the sums' unit
+    const int i = t - (256 - 4 * kTiles), tt = i / 4, q = i % 4;
+    const double u = S.fixed_bad[tt / kSub4] ? 1.0 : pow2d(-2 - S.hsc[tt / kSub4].k0);
+    fit_cubic4<double>(u * S.fn[tt][0][q], u * S.fn[tt][1][q], u * S.fn[tt][2][q], u * S.fn[tt][3][q], S.fq[tt][q]);
   }
   __syncthreads();
-  if (!fixed) {
-    wave_samples_f64(iv, bq, fq, g, j0, kfirst, jplunge, span, dt, t0, ks, n_max, scale, exact_f, z);
-    return;
-  }
-  const int lks = __ffs(ks) - 1;   // ks: a power of two
   const double so = (double)t * (1.0 / kTile);
   const double inv_ks = 1.0 / (double)ks;
 #pragma unroll 1
   for (int tt = 0; tt < kTiles; ++tt) {
-    const int r = tt * kTile + t;   // offset in the segment
-    const int64_t j = j0 + r;
+    const int sub = tt / kSub4;
+    if (S.fixed_bad[sub]) {
+      const int64_t js = j0 + sub * kSegF;
+      wave_samples_f64(S.iv, S.bq[sub], S.fq + sub * kSub4, S.g, js, kfirst, jplunge, tile_span(js, jplunge, kSegF), dt,
+                       t0, ks, n_max, scale, exact_f, z);
+      tt += kSub4 - 1;
+      continue;
+    }
+    const int rc = tt * kTile + t;     // offset in the CTA's samples
+    const int64_t j = j0 + rc;
     double2 out = make_double2(0.0, 0.0);
     if (j < jplunge) {
-      const int ki = ks >= kSegF ? 0 : r >> lks;
-      const int tau = ks >= kSegF ? r : r & (ks - 1);
-      const int s31 = tau << (31 - lks);
-      const IvX& v = ivx[ki];
+      const int ki = rc >> lks, tau = rc & (ks - 1), s31 = tau << (31 - lks);
+      const IvX& v = S.ivx[ki];
+      const HarmX* hx = S.hx[sub];
+      const int sh1 = S.hsc[sub].sh1, sh2 = S.hsc[sub].sh2, r = rc & (kSegF - 1);
       fx::i64 Cs, Ss, Rs, Hp, Hx;
-      const fx::Trig ph = fx::sincos_cycles(phase_at(v.ph, tau, s31), ex);
-      if (hsc.two) harmonics_fixed<true>(ph, r, hx, n_max, hsc.sh1, hsc.sh2, Cs, Ss, Rs);
-      else harmonics_fixed<false>(ph, r, hx, n_max, hsc.sh1, hsc.sh2, Cs, Ss, Rs);
-      response_fixed(gx, fx::sincos_cycles(phase_at(v.gm, tau, s31), ex),
-                     fx::sincos_cycles(phase_at(v.al, tau, s31), ex), Cs, Ss, Rs, Hp, Hx);
-      const double A = poly3<double>(iv[ki].am, (double)tau * inv_ks);
+      const fx::Trig ph = fx::sincos_cycles(phase_at(v.ph, tau, s31), S.ex);
+      if (S.hsc[sub].two) harmonics_fixed<true>(ph, r, hx, n_max, sh1, sh2, Cs, Ss, Rs);
+      else harmonics_fixed<false>(ph, r, hx, n_max, sh1, sh2, Cs, Ss, Rs);
+      response_fixed(S.gx, fx::sincos_cycles(phase_at(v.gm, tau, s31), S.ex),
+                     fx::sincos_cycles(phase_at(v.al, tau, s31), S.ex), Cs, Ss, Rs, Hp, Hx);
+      const double A = poly3<double>(S.iv[ki].am, (double)tau * inv_ks);
       double F[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) F[q] = cubic_at<double>(fq[tt][q], so);
+      for (int q = 0; q < 4; ++q) F[q] = cubic_at<double>(S.fq[tt][q], so);
       const double hp = (double)Hp, hc = (double)Hx;
       out = make_double2(A * (F[0] * hp + F[1] * hc), A * (F[2] * hp + F[3] * hc));
     }
@@ -1026,39 +1038,45 @@ __global__ void __launch_bounds__(kTile, 2) k2_wave_f64(const Knot* __restrict__
   }
 }
 
-// Mixed kernel: one CTA per segment of kSegM = 1024, 2048 or 4096 samples
-// (tiles of 256, four per pass of the sample loop: each thread evaluates the
-// samples at its offset in four tiles at once, four CTAs per SM at 64
-// registers: as fast as three at 78 alone, and one CTA's registers then hold
-// a pass-2 CTA of the pipelined schedule), so the Bessel amplitude
-// fit -- a quadratic in time per harmonic, from three nodes -- is made once
-// per segment.  The eccentricity moves by ~1e-4 relative per 256 samples, and
-// the fit's error grows as the cube of the segment: ~5e-14 of the amplitudes
-// over 2048 samples, far below FP32 resolution.  Longer segments spend less
-// of the kernel in that set-up (its barrier waits); the launch takes the
-// length from the series length alone (at least 16 segments per walker).
+// Mixed kernel: one CTA per segment of kSegM = 1024, 2048 or 4096 samples, with
+// the Bessel amplitude fit -- a quadratic in time per harmonic, from three
+// nodes -- made once per segment.  The eccentricity moves by ~1e-4 relative per
+// 256 samples, and the fit's error grows as the cube of the segment: ~5e-14 of
+// the amplitudes over 2048 samples, far below FP32 resolution.  Longer
+// segments spend less of the kernel in that set-up (its barrier waits); the
+// launch takes the length from the series length alone (at least 16 segments
+// per walker).
+//
+// A warp takes blocks of 128 samples, four per lane: the lanes first reduce the
+// quadratics to the block (a lane per harmonic), where their curvature, ~2^-12
+// of the segment's, is below FP32 resolution except close to a plunge
+// (`curved`), so a harmonic takes 8 paired FMAs per pair of samples instead
+// of 11 and three 16-byte loads instead of five; the samples of a pair lie 32
+// apart in one knot interval, and share its record, the pattern cubics and the phase's 64-bit product.  Bound
+// by the FMA pipe (99 paired and ~170 other instructions a sample at n_max =
+// 20; 114 paired with the quadratics evaluated per sample, 35.0 -> 33.8 ms for
+// 1024 walkers x 2^21).  Four CTAs per SM at 64 registers (three at 80: the
+// same).
 //
 // exact_f: exact patterns per sample (long sample intervals), dphib: the
 // LISA orbital phase step per sample [cycles] for them.  No FP64 instruction
 // runs per thread: e0 is tested once per CTA.
-template <int kSegM, bool kOneIv>
+template <int kSegM>
 __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
                                                           int64_t n, int exact_f, float dphib, int ks, int n_max,
                                                           float2* __restrict__ z, int unit_scale,
                                                           const float* __restrict__ bc, const float* __restrict__ ifact,
                                                           const double* __restrict__ lisa, const IvM* __restrict__ ivs) {
+  constexpr int kTiles = kSegM / kTile;
   __shared__ IvM iv[kSegM / 64];
   __shared__ float bnode[3 * 32 * 3];
-  __shared__ __align__(16) float bq[32 * kAmpStrideM];
-  constexpr int kTiles = kSegM / kTile;
-  static_assert(kTiles % 4 == 0, "tiles are processed in fours");
+  __shared__ __align__(16) float bq[32 * kQuadStride];
+  __shared__ BlkAmp amps[kTile / 32][32];
   __shared__ float fn[kTiles][4][4];   // the four patterns at the fit nodes of each tile
-  // their cubics in (t mod 256) / 256, tiles paired: fq2[m][q][k] = (tile 2m, tile 2m + 1)
-  __shared__ __align__(16) float2 fq2[kTiles / 2][4][4];
+  __shared__ __align__(16) float2 fq[kTiles][4][4];   // their cubics in (t mod 256) / 256, each coefficient twice
   __shared__ float cs0[kTiles][2];     // cos, sin phibar at each tile's start
   __shared__ Geo<float> g;
   __shared__ float4 gk[5];             // response_pair's duplicated geometry constants
-  __shared__ int64_t jplunge;
   __shared__ int cheb_s;
   const int wk = blockIdx.y;
   const WalkerC& C = wcs[wk];
@@ -1066,10 +1084,12 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
   const int64_t j0 = (int64_t)blockIdx.x * kSegM;
   const int64_t kfirst = j0 / ks;
   const int ni = ks >= kSegM ? 1 : kSegM / ks;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, lane = t & 31, wq = t >> 5;
   const float scale = unit_scale ? C.gf.amp_scale : 1.f;
-  if (C.j_plunge <= j0) {   // nothing left of the inspiral
-    for (int r = t; r < kSegM; r += kTile) z[(int64_t)wk * n + j0 + r] = make_float2(0.f, 0.f);
+  const int64_t jplunge = C.j_plunge;
+  z += (int64_t)wk * n + j0;
+  if (jplunge <= j0) {   // nothing left of the inspiral
+    for (int r = t; r < kSegM; r += kTile) z[r] = make_float2(0.f, 0.f);
     return;
   }
   if (t < ni) iv[t] = ivs[(int64_t)wk * nk + kfirst + t];
@@ -1091,7 +1111,6 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
     gk[2] = make_float4(G.cpe1, G.cpe1, G.cpe2, G.cpe2);
     gk[3] = make_float4(G.cqe1, G.cqe1, G.cqe2, G.cqe2);
     gk[4] = make_float4(-G.spS, -G.spS, -G.sqS, -G.sqS);
-    jplunge = C.j_plunge;
     cheb_s = C.e0 < 0.5;
   }
   __syncthreads();
@@ -1099,96 +1118,130 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
     const int i = t - 128, tt = i / 4, q = i % 4;
     float cf[4];
     fit_cubic4<float>(fn[tt][0][q], fn[tt][1][q], fn[tt][2][q], fn[tt][3][q], cf);
-    float* o = reinterpret_cast<float*>(&fq2[tt >> 1][q][0]) + (tt & 1);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) o[2 * k] = cf[k];
+    for (int k = 0; k < 4; ++k) fq[tt][q][k] = make_float2(cf[k], cf[k]);
   }
   const int span = tile_span(j0, jplunge, kSegM);
   const bool cheb = cheb_s != 0;   // per walker (uniform in the CTA)
-  tile_harmonics<float, IvM>(iv, ni, j0, kfirst, ks, n_max, span, bnode, bq, bc, ifact);
+  tile_harmonics(iv, ni, j0, kfirst, ks, n_max, span, bnode, bq, bc, ifact);
   __syncthreads();
   const float inv_span = 1.f / (float)span;
   const float inv_ks = 1.f / (float)ks;
-  const int lks = __ffs(ks) - 1;   // ks is a power of two: the interval index by a shift
+  const int lks = __ffs(ks) - 1;   // ks is a power of two
+  const int jv = (int)(jplunge - j0 < kSegM ? jplunge - j0 : kSegM);   // valid samples of the segment
   constexpr float kTwoPiF = 6.283185307179586f;
-  // per-sample inputs: the orbital phase (for the harmonic sums) first, the
-  // response's angles and amplitude after the sums (fewer registers live
-  // across the harmonic loop)
-  // knot interval ki and offset tau in it of sample r; with K_s >= four
-  // tiles (kOneIv) the four samples of a pass share the interval of the
-  // first, so its record is read once for the four
-  auto interval = [&](const int (&r)[4], int i, int& ki, int& tau) {
-    ki = ks >= kSegM ? 0 : (kOneIv ? r[0] : r[i]) >> lks;
-    tau = r[i] - ki * ks;
-  };
-  auto orb = [&](int ki, int tau, float& cph, float& sph) {
-    const float s = (float)tau * inv_ks;
-    const IvM& v = iv[ki];
-    const float fph = phase_fx(v.ph_base, v.ph_inc, v.ph_c, tau, s);
-    __sincosf(kTwoPiF * fph, &sph, &cph);
-  };
-  auto resp_in = [&](int ki, int tau, float& c2g, float& s2g, float& ca, float& sa, float& A) {
-    const float s = (float)tau * inv_ks;
-    const IvM& v = iv[ki];
-    const float fgm = phase_fx(v.gm_base, v.gm_inc, v.gm_c, tau, s);   // 2 gamma~
-    const float fal = phase_fx(v.al_base, v.al_inc, v.al_c, tau, s);
-    A = poly3<float>(v.am, s);
-    __sincosf(kTwoPiF * fgm, &s2g, &c2g);
-    __sincosf(kTwoPiF * fal, &sa, &ca);
-  };
-  // the four patterns at offset t of tiles tt (even) and tt + 1, paired
-  const float so = (float)t * (1.f / kTile);
-  const float2 so2 = make_float2(so, so);
-  auto patterns2 = [&](int tt, float2 F[4]) {
-    if (!exact_f) {
+  // curvature over half a block against the amplitudes
+  const float* q9 = bq + kQuadStride * lane;   // the lane's harmonic
+  const float half = 0.5f * kBlk * inv_span;
+  float m0 = 0.f, m2 = 0.f;
+  if (lane < n_max) {
+    m0 = fabsf(q9[0]) + fabsf(q9[3]) + fabsf(q9[6]);
+    m2 = fabsf(q9[2]) + fabsf(q9[5]) + fabsf(q9[8]);
+  }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float2* c = fq2[tt >> 1][q];
-        F[q] = __ffma2_rn(__ffma2_rn(__ffma2_rn(c[3], so2, c[2]), so2, c[1]), so2, c[0]);
-      }
-    } else {
-      float sd, cd, FA[4], FB[4];
-      __sincosf(kTwoPiF * dphib * (float)t, &sd, &cd);
-      antenna_fixed<float>(g, cs0[tt][0] * cd - cs0[tt][1] * sd, cs0[tt][1] * cd + cs0[tt][0] * sd, scale, FA);
-      antenna_fixed<float>(g, cs0[tt + 1][0] * cd - cs0[tt + 1][1] * sd, cs0[tt + 1][1] * cd + cs0[tt + 1][0] * sd,
-                           scale, FB);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) F[q] = make_float2(FA[q], FB[q]);
-    }
+  for (int off = 16; off > 0; off >>= 1) {
+    m0 += __shfl_xor_sync(0xffffffffu, m0, off);
+    m2 += __shfl_xor_sync(0xffffffffu, m2, off);
+  }
+  const bool curved = !(m2 * (half * half) < 0x1p-26f * m0);
+  BlkAmp* const amp = amps[wq];
+  const float2 u[2] = {make_float2((float)(lane - 64), (float)(lane - 32)), make_float2((float)lane, (float)(lane + 32))};
+  auto dup = [](float x) { return make_float2(x, x); };
+  // cos, sin of a fixed-point phase (base + inc tau mod 1, plus s^2 (c0 + c1 s))
+  // at tau and tau + 32 [the second 64-bit product is a sum], reduced to half a
+  // cycle by adding and subtracting 1.5 * 2^23
+  auto sincos2 = [&](unsigned long long base, long long inc, const float* c, int tau, float2 s, float2& cs, float2& sn) {
+    const unsigned long long pa = base + (unsigned long long)tau * (unsigned long long)inc;
+    const unsigned long long pb = pa + ((unsigned long long)inc << 5);
+    float2 f = __fmul2_rn(__ffma2_rn(dup(c[1]), s, dup(c[0])), __fmul2_rn(s, s));
+    f = __ffma2_rn(make_float2((float)(int)(unsigned)(pa >> 32), (float)(int)(unsigned)(pb >> 32)),
+                   dup(2.3283064365386963e-10f), f);
+    const float2 r = __fadd2_rn(__fadd2_rn(f, dup(12582912.f)), dup(-12582912.f));
+    f = __fmul2_rn(__fadd2_rn(f, neg2(r)), dup(kTwoPiF));
+    __sincosf(f.x, &sn.x, &cs.x);
+    __sincosf(f.y, &sn.y, &cs.y);
   };
-  // four samples per thread (tiles tt..tt+3, offset t): the amplitude
-  // coefficients of each harmonic are loaded once for all four
 #pragma unroll 1
-  for (int tt = 0; tt < kTiles; tt += 4) {
-    int r[4], ki[4], tau[4];
-    float2 c1[2], s1[2], st[2];
+  for (int rb = wq * kBlk; rb < kSegM; rb += kTile / 32 * kBlk) {
+    if (rb >= jv) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) r[i] = (tt + i) * kTile + t;
+      for (int i = 0; i < 4; ++i) z[rb + 32 * i + lane] = make_float2(0.f, 0.f);
+      continue;
+    }
+    __syncwarp();
+    if (lane < n_max) {
+      const float tc = (float)(rb + kBlk / 2) * inv_span;
+      float A0[3], A1[3], A2[3];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) interval(r, i, ki[i], tau[i]);
+      for (int f = 0; f < 3; ++f) {
+        const float a = fmaf(q9[3 * f + 2], tc, q9[3 * f + 1]);
+        A0[f] = fmaf(a, tc, q9[3 * f]);
+        A1[f] = fmaf(q9[3 * f + 2], tc, a) * inv_span;
+        A2[f] = q9[3 * f + 2] * (inv_span * inv_span);
+      }
+      BlkAmp& o = amp[lane];
+      o.a = make_float4(A0[0], A0[0], A1[0], A1[0]);
+      o.b = make_float4(A0[1], A0[1], A1[1], A1[1]);
+      o.c = make_float4(A0[2], A0[2], A1[2], A1[2]);
+      if (curved) {
+        o.ab2 = make_float4(A2[0], A2[0], A2[1], A2[1]);
+        o.c2 = make_float4(A2[2], A2[2], 0.f, 0.f);
+      }
+    }
+    __syncwarp();
+    // pair p: samples 64 p + lane (x) and 64 p + 32 + lane (y) of the block, in
+    // one knot interval (K_s >= 64)
+    float2 c1[2], s1[2], Cs[2], Ss[2], Rs[2];
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-      float ca_, sa_, cb_, sb_;
-      orb(ki[2 * p], tau[2 * p], ca_, sa_);
-      orb(ki[2 * p + 1], tau[2 * p + 1], cb_, sb_);
-      c1[p] = make_float2(ca_, cb_);
-      s1[p] = make_float2(sa_, sb_);
-      st[p] = make_float2((float)r[2 * p] * inv_span, (float)r[2 * p + 1] * inv_span);
+      const int ki = (rb + 64 * p) >> lks, tau = rb + 64 * p + lane - (ki << lks);
+      const float2 s = make_float2((float)tau * inv_ks, (float)(tau + 32) * inv_ks);
+      const IvM& v = iv[ki];
+      sincos2(v.ph_base, v.ph_inc, v.ph_c, tau, s, c1[p], s1[p]);
     }
-    float2 Cs[2], Ss[2], Rs[2];
-    harmonic_sums4(c1, s1, st, bq, n_max, cheb, Cs, Ss, Rs);
+    if (curved) harmonic_sums4<true>(c1, s1, u, amp, n_max, cheb, Cs, Ss, Rs);
+    else harmonic_sums4<false>(c1, s1, u, amp, n_max, cheb, Cs, Ss, Rs);
+    const int tt = rb / kTile;
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {   // samples r[2p] (x) and r[2p + 1] (y)
-      float2 c2g, s2g, ca, sa, A, F[4], hI, hII;
-      resp_in(ki[2 * p], tau[2 * p], c2g.x, s2g.x, ca.x, sa.x, A.x);
-      resp_in(ki[2 * p + 1], tau[2 * p + 1], c2g.y, s2g.y, ca.y, sa.y, A.y);
-      patterns2(tt + 2 * p, F);
+    for (int p = 0; p < 2; ++p) {
+      const int ki = (rb + 64 * p) >> lks, tau = rb + 64 * p + lane - (ki << lks);
+      const float2 s = make_float2((float)tau * inv_ks, (float)(tau + 32) * inv_ks);
+      const IvM& v = iv[ki];
+      float2 c2g, s2g, ca, sa, F[4], hI, hII;
+      sincos2(v.gm_base, v.gm_inc, v.gm_c, tau, s, c2g, s2g);   // 2 gamma~
+      sincos2(v.al_base, v.al_inc, v.al_c, tau, s, ca, sa);
+      const float2 A = __ffma2_rn(__ffma2_rn(__ffma2_rn(dup(v.am[3]), s, dup(v.am[2])), s, dup(v.am[1])), s, dup(v.am[0]));
+      const int ra = (rb & (kTile - 1)) + 64 * p + lane;      // offsets in the tile: ra, ra + 32
+      if (!exact_f) {
+        const float2 so = make_float2((float)ra * (1.f / kTile), (float)(ra + 32) * (1.f / kTile));
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2* c = fq[tt][q];
+          F[q] = __ffma2_rn(__ffma2_rn(__ffma2_rn(c[3], so, c[2]), so, c[1]), so, c[0]);
+        }
+      } else {
+        float sd, cd, FA[4], FB[4];
+        const float cb = cs0[tt][0], sb = cs0[tt][1];
+        __sincosf(kTwoPiF * dphib * (float)ra, &sd, &cd);
+        antenna_fixed<float>(g, cb * cd - sb * sd, sb * cd + cb * sd, scale, FA);
+        __sincosf(kTwoPiF * dphib * (float)(ra + 32), &sd, &cd);
+        antenna_fixed<float>(g, cb * cd - sb * sd, sb * cd + cb * sd, scale, FB);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) F[q] = make_float2(FA[q], FB[q]);
+      }
       response_pair(gk, c2g, s2g, ca, sa, A, Cs[p], Ss[p], Rs[p], F, hI, hII);
-      const int64_t ja = j0 + r[2 * p], jb = j0 + r[2 * p + 1];
-      z[(int64_t)wk * n + ja] = ja < jplunge ? make_float2(hI.x, hII.x) : make_float2(0.f, 0.f);
-      z[(int64_t)wk * n + jb] = jb < jplunge ? make_float2(hI.y, hII.y) : make_float2(0.f, 0.f);
+      const int r = rb + 64 * p + lane;
+      z[r] = r < jv ? make_float2(hI.x, hII.x) : make_float2(0.f, 0.f);
+      z[r + 32] = r + 32 < jv ? make_float2(hI.y, hII.y) : make_float2(0.f, 0.f);
     }
   }
+}
+
+static bool wave_smem_limits() {
+  return cudaFuncSetAttribute(k2_wave_f64<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(WaveSmem<4>)) ==
+             cudaSuccess &&
+         cudaFuncSetAttribute(k2_wave_f64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(WaveSmem<1>)) ==
+             cudaSuccess;
 }
 
 void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double dt, double t0,
@@ -1201,9 +1254,13 @@ void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double 
     const int ww = w - w0 < kMaxGridY ? w - w0 : kMaxGridY;
     const Knot* kn = knots + (int64_t)w0 * (nk + 1);
     if (o.precision == 0) {
-      dim3 grid((unsigned)(n / kSegF), (unsigned)ww);
-      k2_wave_f64<<<grid, kTile, 0, s>>>(kn, wc + w0, n, dt, t0, o.ks, o.n_max, (double2*)z + (int64_t)w0 * n,
-                                         unit_scale ? 1 : 0, dt > kPatternFitDtMax64 ? 1 : 0, bt.c64, bt.f64, lisa);
+      // four segments a CTA where that still gives every SM four CTAs
+      const int sub = n >= 4 * kSegF && (n / (4 * kSegF)) * ww >= 4 * 152 ? 4 : 1;
+      auto* kern = sub == 4 ? k2_wave_f64<4> : k2_wave_f64<1>;
+      const size_t sm = sub == 4 ? sizeof(WaveSmem<4>) : sizeof(WaveSmem<1>);
+      kern<<<dim3((unsigned)(n / (sub * kSegF)), (unsigned)ww), kTile, sm, s>>>(
+          kn, wc + w0, n, dt, t0, o.ks, o.n_max, (double2*)z + (int64_t)w0 * n, unit_scale ? 1 : 0,
+          dt > kPatternFitDtMax64 ? 1 : 0, bt.c64, bt.f64, lisa);
     } else {
       // segment length from the series length alone (so a walker's result
       // does not depend on the batch it is in): at least 16 segments per
@@ -1215,16 +1272,11 @@ void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double 
       float2* zz = (float2*)z + (int64_t)w0 * n;
       const IvM* iv = (const IvM*)ivs + (int64_t)w0 * nk;
       const int us = unit_scale ? 1 : 0;
-#define EMRI_WAVE_MIXED(SEG, ONE) \
-  k2_wave_mixed<SEG, ONE><<<grid, kTile, 0, s>>>(kn, wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
-      const bool one = o.ks >= 4 * kTile;   // one knot interval per pass of four samples
-      if (seg == 4096) {
-        if (one) EMRI_WAVE_MIXED(4096, true); else EMRI_WAVE_MIXED(4096, false);
-      } else if (seg == 2048) {
-        if (one) EMRI_WAVE_MIXED(2048, true); else EMRI_WAVE_MIXED(2048, false);
-      } else {
-        if (one) EMRI_WAVE_MIXED(1024, true); else EMRI_WAVE_MIXED(1024, false);
-      }
+#define EMRI_WAVE_MIXED(SEG) \
+  k2_wave_mixed<SEG><<<grid, kTile, 0, s>>>(kn, wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
+      if (seg == 4096) EMRI_WAVE_MIXED(4096);
+      else if (seg == 2048) EMRI_WAVE_MIXED(2048);
+      else EMRI_WAVE_MIXED(1024);
 #undef EMRI_WAVE_MIXED
     }
   }
