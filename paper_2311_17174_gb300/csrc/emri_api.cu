@@ -551,8 +551,9 @@ extern "C" int emri_ctx_create(int device, size_t budget, emri_ctx** out) {
   }
   launch_twiddle_init(c->tw, c->stream);
   cudaMemcpyAsync(c->gl, glh, sizeof glh, cudaMemcpyHostToDevice, c->stream);
-  fft_set_smem_limits();
+  const bool fft_ok = fft_setup();
   e2 = cudaStreamSynchronize(c->stream);
+  if (e2 == cudaSuccess && !fft_ok) e2 = cudaErrorUnknown;
   if (e2 == cudaSuccess) e2 = cudaGetLastError();
   if (e2 == cudaSuccess && upload_exp512()) e2 = cudaErrorUnknown;
   if (e2 == cudaSuccess && emri::upload_bessel_tables(c->bt)) e2 = cudaErrorUnknown;

@@ -63,7 +63,7 @@ int upload_exp512();
 
 void launch_prologue(const double* theta, int64_t ld, int w, int64_t n, double dt, const OptsN& o,
                      const double* gl, WalkerC* out, cudaStream_t s);
-// (FP64 tab with n1 >= 256: (cos.h, cos.l, sin.h, sin.l) in Q62, four ints)
+// (FP64 tab with n1 >= 256: (cos.h, cos.l, sin.h, sin.l) in Q62, balanced halves (fx64.cuh), four ints)
 // tab[w][n1] = exp(-2 pi i frac(n2 k1 r)), rtab[w][n2] = exp(-2 pi i frac(k2 r))
 void launch_delay_table(const WalkerC* wc, int w, int n1, int n2, bool fp32, void* tab, void* rtab, cudaStream_t s);
 void launch_prologue_export(const WalkerC* wc, int w, double* out, cudaStream_t s);
@@ -107,7 +107,8 @@ void launch_fft_pass2_ip(const void* y, int w, const FftPlan& p, bool fp32, cons
 // dh_scale / hh_scale undo the dataset's FP32 scaling (1 for FP64)
 void launch_finalize(const double2* partial, int n2, const WalkerC* wc, int w, double dh_scale, double hh_scale,
                      double* lnl, double* dh, double* hh, uint32_t* status, cudaStream_t s);
-void fft_set_smem_limits();
+// shared-memory limits and fixed-point tables on the current device; false on failure
+bool fft_setup();
 
 // dataset preparation: the weighted conjugate spectrum g = w conj(D) and
 // the weights w in the pass-2 order (k2-major), plus FP32 copies scaled by

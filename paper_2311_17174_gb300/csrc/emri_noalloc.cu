@@ -80,8 +80,9 @@ int setup_device(int dev, cudaStream_t s, DevState** out) {
     st.tw.tc64 = (double2*)(t + 4096 * 16 + 1024 * 16 + 4096 * 8 + 1024 * 8);
     st.tw.tt32 = (float2*)(t + 4096 * 16 + 1024 * 16 + 4096 * 8 + 1024 * 8 + 4096 * 16);
     launch_twiddle_init(st.tw, s);
-    fft_set_smem_limits();
+    const bool fft_ok = fft_setup();
     e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && !fft_ok) e = cudaErrorUnknown;
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_err(e, "no-alloc FFT set-up");
     st.scratch = (unsigned char*)sp;

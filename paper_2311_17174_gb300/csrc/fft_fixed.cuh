@@ -6,17 +6,16 @@
 // points each in registers: radix-8 Stockham stages, the last one radix 4 or
 // 2, exchanged through shared memory.  The points come and go in double.
 //
-// Scaling: L = sum |Re x_j| + |Im x_j| bounds every intermediate value and
+// Scaling: L = sum |x_j| (from above) bounds every intermediate value and
 // output of the transform (each is a sum of inputs times unit phases), so with
-// L 2^k < 2^62 nothing overflows, and one exponent per transform serves all
-// stages.  The inputs are rounded at 2^-62 L, i.e. for N samples of equal size
-// at ~2^-52 of one sample, the size of a double's own rounding; the stages' roundings
-// (the same absolute size, on values that have grown by sqrt(8) per stage)
-// add less.  RMS error of a 2^20-point transform of noise: 2.4e-16 relative,
-// against 3.9e-16 in double.
-// 128 walkers x 2^21 (passes of 1024 and 2048 points): pass 1 17.6 -> 3.7 ms,
-// pass 2 with the inner products 23.2 -> 4.2 ms; 23 transforms of 2^19 points
-// 1.49 -> 0.38 ms.
+// L 2^k < 2^62 nothing overflows.  For 1024 points and more that leaves too few
+// bits to the inputs (L ~ N |x|): the first two radix-8 stages, whose values are
+// at most 64 max |x_j|, then run at a finer scale of their own, and the second
+// one rounds to the scale of L.  RMS error, 2^16 to 2^22 points of noise or
+// signal: 0.7e-16 to 1.8e-16 relative, against 2.8e-16 to 3.4e-16 in double.
+// 128 walkers x 2^21 (passes of 1024 and 2048 points): pass 1 17.6 -> 3.9 ms,
+// pass 2 with the inner products 23.2 -> 4.3 ms; 23 transforms of 2^19 points
+// 1.49 -> 0.39 ms.
 // Transforms that hold NaN, infinities, or numbers outside [1e-30, 1e30] in
 // sum take the FP64 Stockham form (their CTA does).
 #pragma once
@@ -31,31 +30,37 @@ using fx::wide;
 // exp(-2 pi i r k / (8 NS)), r = 1..7, k < NS at kBase(NS) + (r - 1) NS + k for
 // NS = 8, 64, 512 (radix-8 stages; radix 4 reads r = 2, 4, 6 and radix 2 r = 4
 // of the same NS), then exp(-2 pi i m / 4096) and exp(-2 pi i m / 2^22); each
-// (cos.h, cos.l, sin.h, sin.l), Q62.
+// (cos.h, cos.l, sin.h, sin.l), Q62 in balanced halves.
 constexpr int kStageLen = 7 * (8 + 64 + 512);
 __host__ __device__ constexpr int kBase(int ns) { return ns - 8; }   // 7 (8 + ... + NS/8)
 __device__ int4 g_stage[kStageLen];
 __device__ int4 g_ta[4096];
 __device__ int4 g_tb[1024];
 
-__device__ __forceinline__ int4 pack_unit(double turns) {   // exp(-2 pi i turns)
-  double s, c;
-  sincospi(-2.0 * turns, &s, &c);
-  const Op a = fx::op(llrint(c * 0x1p62)), b = fx::op(llrint(s * 0x1p62));
+FX_HD int4 pack(i64 c, i64 s) {
+  const Op a = fx::bal(c), b = fx::bal(s);
   return make_int4(a.h, a.l, b.h, b.l);
 }
 
-// The tables hold the same values for every context of a device, so a second
-// context's fill rewrites them unchanged.
-__global__ void k_init() {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < kStageLen) {
-    const int ns = i < 56 ? 8 : i < 504 ? 64 : 512;
-    const int j = i - kBase(ns), r = j / ns + 1, k = j % ns;
-    g_stage[i] = pack_unit((double)(r * k) / (double)(8 * ns));
-  }
-  if (i < 4096) g_ta[i] = pack_unit((double)i / 4096.0);
-  if (i < 1024) g_tb[i] = pack_unit((double)i / 4194304.0);
+// Fills the tables of the current device from long double values (a second
+// context's upload rewrites them unchanged).
+static bool upload_tables() {
+  static const std::vector<int4> host = [] {
+    std::vector<int4> t;
+    auto put = [&](long double turns) {
+      const long double x = -2.0L * 3.141592653589793238462643383279502884L * turns;
+      t.push_back(pack(llrintl(cosl(x) * 0x1p62L), llrintl(sinl(x) * 0x1p62L)));
+    };
+    for (int ns = 8; ns <= 512; ns *= 8)
+      for (int r = 1; r < 8; ++r)
+        for (int k = 0; k < ns; ++k) put((long double)(r * k) / (8 * ns));
+    for (int i = 0; i < 4096; ++i) put((long double)i / 4096);
+    for (int i = 0; i < 1024; ++i) put((long double)i / 4194304);
+    return t;
+  }();
+  return cudaMemcpyToSymbol(g_stage, host.data(), sizeof(g_stage)) == cudaSuccess &&
+         cudaMemcpyToSymbol(g_ta, host.data() + kStageLen, sizeof(g_ta)) == cudaSuccess &&
+         cudaMemcpyToSymbol(g_tb, host.data() + kStageLen + 4096, sizeof(g_tb)) == cudaSuccess;
 }
 
 struct Z {
@@ -65,23 +70,30 @@ struct Z {
 FX_HD Z add(Z a, Z b) { return Z{a.x + b.x, a.y + b.y}; }
 FX_HD Z sub(Z a, Z b) { return Z{a.x - b.x, a.y - b.y}; }
 
-// high*high + cross of two products, x 4 (Q62 factor: the unit stays), to the
-// last bit
-FX_HD i64 get4(const Sum& s) { return (s.h << 2) + (s.c >> 29); }
-FX_HD Sum sum4() {
-  Sum s;
-  s.c = (i64)1 << 28;
-  return s;
-}
+// A sum of products in two accumulators, high*high and cross terms (2^32 below
+// it).
+struct Acc {
+  i64 h, c;
+  FX_HD void add(Op a, Op b) {
+    h = wide(a.h, b.h, h);
+    c = wide(a.h, b.l, c);
+    c = wide(a.l, b.h, c);
+  }
+};
+constexpr i64 kHalf4 = (i64)1 << 29;   // half of the last bit of get4
+// x 2^-62 (Q62 factor: the unit stays), rounded to the last bit
+FX_HD i64 get4(const Acc& s) { return (s.h << 2) + (s.c >> 30); }
 
-// a w, w = (cos.h, cos.l, sin.h, sin.l) in Q62, |a| < 2^62
+// a w, w = (cos.h, cos.l, sin.h, sin.l) in Q62, |a| < 2^62: error ~0.55 of the
+// last bit (rms; low*low 0.47, the rounding 0.29).  With op()'s halves it was
+// ~1.7, the larger part of a transform's error.
 FX_HD Z cmul(Z a, int4 w) {
-  const Op ax = fx::op(a.x), ay = fx::op(a.y), c{w.x, w.y}, s{w.z, w.w};
-  Sum re = sum4(), im = sum4(), t = sum4();
+  const Op ax = fx::bal(a.x), ay = fx::bal(a.y), c{w.x, w.y}, s{w.z, w.w};
+  Acc re{0, kHalf4}, im{0, kHalf4}, t{0, 0};
   re.add(ax, c);
   t.add(ay, s);
   re.h -= t.h;
-  re.c -= t.c - ((i64)1 << 28);
+  re.c -= t.c;
   im.add(ax, s);
   im.add(ay, c);
   return Z{get4(re), get4(im)};
@@ -89,8 +101,9 @@ FX_HD Z cmul(Z a, int4 w) {
 
 // x sqrt(1/2) = x - x (1 - sqrt(1/2)), the factor 0.29289... in Q64
 FX_HD i64 mul_h(i64 x) {
-  const i64 k = 0x4AFB0CCC06219B7CLL;
-  return x - fx::mul(fx::op(x), fx::op(k));
+  Acc s{0, (i64)1 << 31};
+  s.add(fx::bal(x), Op{0x4AFB0CCC, 0x06219B7C});
+  return x - (s.h + (s.c >> 32));
 }
 
 FX_HD void dft4(Z& a0, Z& a1, Z& a2, Z& a3) {
@@ -175,9 +188,18 @@ struct Cfg {
 template <int NB>
 __device__ __forceinline__ int at(int i, int c) { return (i + (i >> 3)) * NB + c; }
 
+// Exponent of a transform's values: 2^k from the inputs to the second stage,
+// 2^(k - down) after it.
+struct Scale {
+  int k, down;
+  __device__ __forceinline__ int out() const { return k - down; }
+};
+// From this length on the second stage changes the scale.
+constexpr int kTwoScales = 10;
+
 // v (point t + q T in slot q) -> bin t + q T in slot q.  xb: Cfg::kSmem bytes.
 template <int LG, int NB, int NS>
-__device__ __forceinline__ void stages(Z (&v)[8], longlong2* xb, int t, int c) {
+__device__ __forceinline__ void stages(Z (&v)[8], longlong2* xb, int t, int c, int down) {
   constexpr int N = 1 << LG, T = N / 8;
   if constexpr (8 * NS <= N) {
     const int k = t & (NS - 1);
@@ -186,6 +208,11 @@ __device__ __forceinline__ void stages(Z (&v)[8], longlong2* xb, int t, int c) {
       for (int q = 1; q < 8; ++q) v[q] = cmul(v[q], __ldg(g_stage + kBase(NS) + (q - 1) * NS + k));
     }
     dft8(v);
+    if constexpr (NS == 8 && LG >= kTwoScales) {
+      const i64 half = down ? (i64)1 << (down - 1) : 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = Z{(v[q].x + half) >> down, (v[q].y + half) >> down};
+    }
     if constexpr (8 * NS < N) {
       const int d = (t / NS) * NS * 8 + k;
       if constexpr (NS > 1) __syncthreads();   // the previous stage's reads
@@ -197,7 +224,7 @@ __device__ __forceinline__ void stages(Z (&v)[8], longlong2* xb, int t, int c) {
         const longlong2 u = xb[at<NB>(t + q * T, c)];
         v[q] = Z{u.x, u.y};
       }
-      stages<LG, NB, 8 * NS>(v, xb, t, c);
+      stages<LG, NB, 8 * NS>(v, xb, t, c, down);
     }
   } else if constexpr (4 * NS == N) {   // butterflies t and t + T over v[0,2,4,6] and v[1,3,5,7]
 #pragma unroll
@@ -220,36 +247,52 @@ __device__ __forceinline__ void stages(Z (&v)[8], longlong2* xb, int t, int c) {
 }
 
 // Loads the thread's points p[q T gs] of its transform, finds the transform's
-// exponent and converts.  Returns false, for the whole CTA, when a transform is
-// outside the fixed-point range; otherwise k is the exponent.  swap: exchange
+// exponents and converts.  Returns false, for the whole CTA, when a transform is
+// outside the fixed-point range.  swap: exchange
 // Re and Im (the inverse transform is the forward one of the exchanged parts).
 template <int LG, int NB>
-__device__ __forceinline__ bool load(const double2* p, int64_t step, bool swap, int c, Z (&v)[8], int& k) {
+__device__ __forceinline__ bool load(const double2* p, int64_t step, bool swap, int c, Z (&v)[8], Scale& sc) {
   using F = Cfg<LG, NB>;
   constexpr int NW = F::kThreads / 32;
-  __shared__ float red[NW][NB];
+  __shared__ float red[NW][NB], redm[NW][NB];
   double2 u[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) u[q] = p[q * step];
-  float L = 0.f;
+  float L = 0.f, M = 0.f;
   unsigned any = 0;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    L += abs_float(u[q].x) + abs_float(u[q].y);
+    // |z| <= max + (sqrt(2) - 1) min of the parts' sizes
+    const float a = abs_float(u[q].x), b = abs_float(u[q].y);
+    const float r = fmaf(0.41422f, fminf(a, b), fmaxf(a, b));
+    L += r;
+    M = fmaxf(M, r);
     any |= (unsigned)__double2hiint(u[q].x) << 1 | (unsigned)__double2loint(u[q].x) |
            (unsigned)__double2hiint(u[q].y) << 1 | (unsigned)__double2loint(u[q].y);
   }
 #pragma unroll
-  for (int off = 16; off >= NB; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
-  if ((threadIdx.x & 31) < NB) red[threadIdx.x >> 5][c] = L;
+  for (int off = 16; off >= NB; off >>= 1) {
+    L += __shfl_xor_sync(0xffffffffu, L, off);
+    if (LG >= kTwoScales) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+  }
+  if ((threadIdx.x & 31) < NB) {
+    red[threadIdx.x >> 5][c] = L;
+    if (LG >= kTwoScales) redm[threadIdx.x >> 5][c] = M;
+  }
   const int nonzero = __syncthreads_or(any != 0);   // also orders red
   L = 0.f;
 #pragma unroll 8
-  for (int w = 0; w < NW; ++w) L += red[w][c];
+  for (int w = 0; w < NW; ++w) {
+    L += red[w][c];
+    if (LG >= kTwoScales) M = fmaxf(M, redm[w][c]);
+  }
   const bool bad = !(L < 1e30f) || (L < 1e-30f && nonzero);
   // NB transforms share the decision (each thread sees its own transform's L)
   if (__syncthreads_or(bad)) return false;
-  k = 61 - ilogbf(fmaxf(L * 1.001f, 1e-30f));
+  L = fmaxf(L * 1.001f, 1e-30f);
+  sc.k = 61 - ilogbf(LG >= kTwoScales ? fminf(L, fmaxf(64.064f * M, 1e-30f)) : L);
+  sc.down = sc.k - (61 - ilogbf(L));
+  const int k = sc.k;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const i64 a = to_fixed(u[q].x, k), b = to_fixed(u[q].y, k);
@@ -271,15 +314,9 @@ __device__ __noinline__ void fallback(const double2* p, int64_t step, double2* b
 }
 
 // exp(-2 pi i m / 2^22), m < 2^22
-__device__ __forceinline__ Z twiddle(uint32_t m) {
-  const int4 a = __ldg(g_ta + (m >> 10));
-  const Z za{((i64)a.x << 32) | ((i64)a.y << 1), ((i64)a.z << 32) | ((i64)a.w << 1)};
-  return cmul(za, __ldg(g_tb + (m & 1023u)));
-}
-__device__ __forceinline__ int4 pack(Z w) {
-  const Op c = fx::op(w.x), s = fx::op(w.y);
-  return make_int4(c.h, c.l, s.h, s.l);
-}
+__device__ __forceinline__ Z unit(int4 w) { return Z{fx::value(Op{w.x, w.y}), fx::value(Op{w.z, w.w})}; }
+__device__ __forceinline__ Z twiddle(uint32_t m) { return cmul(unit(__ldg(g_ta + (m >> 10))), __ldg(g_tb + (m & 1023u))); }
+__device__ __forceinline__ int4 pack(Z w) { return pack(w.x, w.y); }
 
 __device__ __forceinline__ double2 out2(Z v, int k, bool swap) {
   const double a = from_fixed(v.x, k), b = from_fixed(v.y, k);
@@ -306,8 +343,8 @@ __global__ void __launch_bounds__(Cfg<LG, NB>::kThreads, 3)
   const bool swap = sign > 0;
   if (threadIdx.x < 8 * NB) sq[t][c] = pack(twiddle((uint32_t)(j1 * F::T * t) << shift22));   // slot t
   Z v[8];
-  int k;
-  if (!load<LG, NB>(zw + (int64_t)t * n1, (int64_t)F::T * n1, swap, c, v, k)) {
+  Scale sc;
+  if (!load<LG, NB>(zw + (int64_t)t * n1, (int64_t)F::T * n1, swap, c, v, sc)) {
     double2* buf = reinterpret_cast<double2*>(smraw);
     fallback<LG, NB>(zw + (int64_t)t * n1, (int64_t)F::T * n1, buf, t, c, sign, tc);
 #pragma unroll 1
@@ -318,12 +355,12 @@ __global__ void __launch_bounds__(Cfg<LG, NB>::kThreads, 3)
     }
     return;
   }
-  stages<LG, NB, 1>(v, xb, t, c);
+  stages<LG, NB, 1>(v, xb, t, c, sc.down);
   const Z w0 = twiddle((uint32_t)(j1 * t) << shift22);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const Z w = q == 0 ? w0 : cmul(w0, sq[q][c]);
-    zo[(int64_t)n1 * (t + q * F::T)] = out2(cmul(v[q], pack(w)), k, swap);
+    zo[(int64_t)n1 * (t + q * F::T)] = out2(cmul(v[q], pack(w)), sc.out(), swap);
   }
 }
 
@@ -341,21 +378,21 @@ __global__ void __launch_bounds__(Cfg<LG, NB>::kThreads, Cfg<LG, NB>::kThreads >
   double2* o = out + (int64_t)blockIdx.y * n + k2;
   const bool swap = sign > 0;
   Z v[8];
-  int k;
-  if (!load<LG, NB>(row, F::T, swap, c, v, k)) {
+  Scale sc;
+  if (!load<LG, NB>(row, F::T, swap, c, v, sc)) {
     double2* buf = reinterpret_cast<double2*>(smraw);
     fallback<LG, NB>(row, F::T, buf, t, c, sign, tc);
 #pragma unroll 1
     for (int q = 0; q < 8; ++q) o[(int64_t)n2 * (t + q * F::T)] = buf[(t + q * F::T) * NB + c];
     return;
   }
-  stages<LG, NB, 1>(v, reinterpret_cast<longlong2*>(smraw), t, c);
+  stages<LG, NB, 1>(v, reinterpret_cast<longlong2*>(smraw), t, c, sc.down);
 #pragma unroll
-  for (int q = 0; q < 8; ++q) o[(int64_t)n2 * (t + q * F::T)] = out2(v[q], k, swap);
+  for (int q = 0; q < 8; ++q) o[(int64_t)n2 * (t + q * F::T)] = out2(v[q], sc.out(), swap);
 }
 
 // Pass 2 of row k2 fused with the inner products.  dtab: the walker's delay
-// factors as (cos.h, cos.l, sin.h, sin.l) in Q62.
+// factors as (cos.h, cos.l, sin.h, sin.l), Q62 in balanced halves.
 //
 // The bin, its product with the delay factor and its square modulus stay in
 // fixed point, normalised per bin so that small bins keep 60 bits; three
@@ -378,10 +415,11 @@ __global__ void __launch_bounds__(Cfg<LG, 1>::kThreads, Cfg<LG, 1>::kThreads > 2
   const double* ws = wperm + base;
   const int4* ts = dtab + (int64_t)wk * F::N;
   Z v[8];
-  int k = 0;
-  const bool fixed = load<LG, 1>(row, F::T, false, 0, v, k);
-  if (fixed) stages<LG, 1, 1>(v, reinterpret_cast<longlong2*>(smraw), t, 0);
+  Scale sc{0, 0};
+  const bool fixed = load<LG, 1>(row, F::T, false, 0, v, sc);
+  if (fixed) stages<LG, 1, 1>(v, reinterpret_cast<longlong2*>(smraw), t, 0, sc.down);
   else fallback<LG, 1>(row, F::T, buf, t, 0, -1, tc);
+  const int k = sc.out();
   const double2 cnv = make_double2(wcs[wk].cn_re, wcs[wk].cn_im);
   double zr = 0.0, zi = 0.0, shh = 0.0;
   if (fixed && !FD) {
@@ -418,7 +456,7 @@ __global__ void __launch_bounds__(Cfg<LG, 1>::kThreads, Cfg<LG, 1>::kThreads > 2
       const double2 H = fixed ? out2(vq, k, false) : buf[k1];
       const int4 w = __ldg(ts + k1);
       const double2 G = __ldg(ds + k1);
-      double2 P = ::emri::cmul(H, out2(Z{((i64)w.x << 32) | ((i64)w.y << 1), ((i64)w.z << 32) | ((i64)w.w << 1)}, 62, false));
+      double2 P = ::emri::cmul(H, out2(unit(w), 62, false));
       if (2 * k1 == F::N && k2 > 0) P = ::emri::cmul(P, cnv);
       double A2 = 1.0;
       if (FD) {

@@ -71,6 +71,12 @@ FX_HD i64 mul(Op a, Op b) {
   return s.get();
 }
 
+// Operand with a signed low half: value = h 2^32 + l, |l| <= 2^31.  One
+// instruction more than op(), but no bit is dropped and low*low averages to
+// zero and stays below 2^62.
+FX_HD Op bal(i64 v) { return Op{(int)((v + 0x80000000LL) >> 32), (int)(uint32_t)v}; }
+FX_HD i64 value(Op a) { return ((i64)a.h << 32) + a.l; }
+
 // a f 2^-32 for 0 <= f < 2^31
 FX_HD i64 mul31(i64 a, int f) {
   const u64 l = wideu(lo(a), (uint32_t)f, 0);

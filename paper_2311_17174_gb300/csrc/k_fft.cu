@@ -25,6 +25,10 @@
 #include "emri_internal.h"
 #include "fx64.cuh"
 
+#include <math.h>
+#include <string.h>
+#include <vector>
+
 namespace emri {
 
 constexpr int kFftThreads = 512;   // pass 1 (column groups)
@@ -82,11 +86,8 @@ __global__ void k_twiddle_init(double2* ta64, double2* tb64, float2* ta32, float
   }
 }
 
-static void launch_fixed_twiddles(cudaStream_t s);
-
 void launch_twiddle_init(Twiddles t, cudaStream_t s) {
   k_twiddle_init<<<16, 256, 0, s>>>(t.ta64, t.tb64, t.ta32, t.tb32, t.tc64, t.tt32);
-  launch_fixed_twiddles(s);
 }
 
 // ----------------------------------------------------- complex helpers
@@ -660,6 +661,69 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(C2) == 8 ? 2 : 1) k3_pass1
   }
 }
 
+// FP32 columns of 256 or 512 points in registers (r8), NB adjacent columns by
+// NB N2/8 threads: the points come straight from global memory and leave with
+// the inter-pass twiddle (W^{j1 t} of the thread times W^{j1 T q}, one per
+// column and slot), so shared memory carries only the stages' exchanges.
+// Element i of column c at (i + i/8) NB + c: the eight-point writes of the
+// first stage fall into different banks.  333 walkers x 2^18 (512 points):
+// 0.367 -> 0.313 ms against the shared-memory tile of k3_pass1, which stays for
+// 1024 points: there eight columns take 1024 threads and four read 32-byte
+// pieces of the rows, 11.2 and 10.2 against 7.9 ms (1024 walkers x 2^21).
+// The inverse transform is the forward one with Re and Im exchanged.
+template <int LG, int NB, int S>
+__device__ __forceinline__ void col_stages8(float2 (&v)[8], float2* xb, const float2* __restrict__ tt, int t, int c) {
+  constexpr int N = 1 << LG, T = N / 8, NS = 1 << (3 * S);
+  if constexpr (8 * NS <= N) {
+    const int k = t & (NS - 1);
+    if constexpr (NS > 1) r8::twiddle8(v, tt[4 * NS + k]);
+    r8::dft8(v);
+    if constexpr (8 * NS < N) {
+      auto at = [&](int i) { return (i + (i >> 3)) * NB + c; };
+      const int d = (t / NS) * NS * 8 + k;
+      if constexpr (NS > 1) __syncthreads();   // the previous stage's reads
+#pragma unroll
+      for (int q = 0; q < 8; ++q) xb[at(d + q * NS)] = v[q];
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = xb[at(t + q * T)];
+      col_stages8<LG, NB, S + 1>(v, xb, tt, t, c);
+    }
+  }
+}
+
+template <int LG, int NB>
+constexpr size_t col_smem() {
+  return (size_t)NB * ((1 << LG) + (1 << LG) / 8) * sizeof(float2);
+}
+
+template <int LG, int NB>
+__global__ void __launch_bounds__(NB * (1 << LG) / 8)
+    k3_pass1_r8(const float2* zin, float2* zout, int64_t n, int n1, int sign, int shift22,
+                const float2* __restrict__ ta, const float2* __restrict__ tb, const float2* __restrict__ tt) {
+  constexpr int T = (1 << LG) / 8;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ float2 sq[8][NB];
+  const int c = threadIdx.x % NB, t = threadIdx.x / NB;
+  const int j1 = blockIdx.x * NB + c;
+  const int64_t col = (int64_t)blockIdx.y * n + j1;
+  if (threadIdx.x < 8 * NB) sq[t][c] = twiddle22(ta, tb, (uint32_t)(j1 * T * t) << shift22, -1);
+  float2 v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float2 u = zin[col + (int64_t)n1 * (t + q * T)];
+    v[q] = sign > 0 ? make_float2(u.y, u.x) : u;
+  }
+  col_stages8<LG, NB, 0>(v, reinterpret_cast<float2*>(smraw), tt, t, c);
+  r8::last_stage<LG>(v, tt, t);
+  const float2 w0 = twiddle22(ta, tb, (uint32_t)(j1 * t) << shift22, -1);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float2 u = r8::mul(v[q], q == 0 ? w0 : r8::mul(w0, sq[q][c]));
+    zout[col + (int64_t)n1 * (t + q * T)] = sign > 0 ? make_float2(u.y, u.x) : u;
+  }
+}
+
 // --------------------------------------------------- pass 2, natural order
 // Rows of up to 128 points (FP64: fft_fixed.cuh from 256 on; FP32: below)
 template <typename C2, int LG>
@@ -1117,11 +1181,8 @@ static void pass1_dispatch(const C2* z, C2* out, int batch, const FftPlan& p, in
   if (lg == 5) pass1_inst<C2, NB, 5>(z, out, batch, p, sign, shift, ta, tb, tf, s);
   if (lg == 6) pass1_inst<C2, NB, 6>(z, out, batch, p, sign, shift, ta, tb, tf, s);
   if (lg == 7) pass1_inst<C2, NB, 7>(z, out, batch, p, sign, shift, ta, tb, tf, s);
-  if constexpr (sizeof(C2) == sizeof(float2)) {   // FP64 columns of 256 points and more: pass1_fixed
-    if (lg == 8) pass1_inst<C2, NB, 8>(z, out, batch, p, sign, shift, ta, tb, tf, s);
-    if (lg == 9) pass1_inst<C2, NB, 9>(z, out, batch, p, sign, shift, ta, tb, tf, s);
-    if (lg >= 10) pass1_inst<C2, NB, 10>(z, out, batch, p, sign, shift, ta, tb, tf, s);
-  }
+  if constexpr (sizeof(C2) == sizeof(float2))
+    if (lg == 10) pass1_inst<C2, NB, 10>(z, out, batch, p, sign, shift, ta, tb, tf, s);
 }
 
 static int log2i(int v) {
@@ -1130,8 +1191,6 @@ static int log2i(int v) {
   return lg;
 }
 
-
-static void launch_fixed_twiddles(cudaStream_t s) { fxfft::k_init<<<16, 256, 0, s>>>(); }
 
 // FP64 columns of 256, 512, 1024 points: fixed point, 256 threads a CTA
 template <int LG>
@@ -1142,10 +1201,21 @@ static void pass1_fixed(const double2* z, double2* out, int batch, const FftPlan
       z, out, p.n, p.n1, sign, 22 - p.log2n, t.ta64, t.tb64, t.tc64);
 }
 
+template <int LG, int NB>
+static void pass1_r8(const float2* z, float2* out, int batch, const FftPlan& p, int sign, const Twiddles& t,
+                     cudaStream_t s) {
+  k3_pass1_r8<LG, NB><<<dim3(p.n1 / NB, batch), NB * (1 << LG) / 8, col_smem<LG, NB>(), s>>>(
+      z, out, p.n, p.n1, sign, 22 - p.log2n, t.ta32, t.tb32, t.tt32);
+}
+
 void launch_fft_pass1(const void* z, void* out, int batch, const FftPlan& p, bool fp32, int sign, const Twiddles& t,
                       cudaStream_t s) {
   if (batch <= 0) return;
-  if (fp32)
+  if (fp32 && p.n2 == 512)
+    pass1_r8<9, 8>((const float2*)z, (float2*)out, batch, p, sign, t, s);
+  else if (fp32 && p.n2 == 256)
+    pass1_r8<8, 8>((const float2*)z, (float2*)out, batch, p, sign, t, s);
+  else if (fp32)
     pass1_dispatch<float2, FftCfg<float2>::kCols>((const float2*)z, (float2*)out, batch, p, sign, t.ta32, t.tb32, t.ta32, s);
   else if (p.n2 >= 1024)
     pass1_fixed<10>((const double2*)z, (double2*)out, batch, p, sign, t, s);
@@ -1284,20 +1354,20 @@ void launch_inner_dd(const double2* d, const double* w, int64_t n, double* out, 
   k_inner_dd<<<1, 1024, 0, s>>>(d, w, n, out);
 }
 
-// Raise the dynamic shared-memory limit of the FFT kernels (once per device).
+// Raises the dynamic shared-memory limit of the FFT kernels and uploads the
+// fixed-point tables (once per device); false on failure.
 template <typename F>
 static void raise(F f) {
   cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
-void fft_set_smem_limits() {
-#define P1(L) raise(k3_pass1<float2, L, FftCfg<float2>::kCols>)
-  P1(5); P1(6); P1(7); P1(8); P1(9); P1(10);
-#undef P1
+bool fft_setup() {
+  raise(k3_pass1_r8<8, 8>), raise(k3_pass1_r8<9, 8>);
+  raise(k3_pass1<float2, 10, FftCfg<float2>::kCols>);
   raise(k4_pass2_store<float2, 5>), raise(k4_pass2_store<float2, 6>), raise(k4_pass2_store<float2, 7>);
   raise(k4_pass2_store_r8<8, 8>), raise(k4_pass2_store_r8<9, 4>), raise(k4_pass2_store_r8<10, 4>);
   raise(k4_pass2_store_r8<11, 4>), raise(k4_pass2_store_r8<12, 2>);
-#define P2S(L) raise(k3_pass1<double2, L, FftCfg<double2>::kCols>), raise(k4_pass2_store<double2, L>),       \
+#define P2S(L) raise(k3_pass1<double2, L, FftCfg<double2>::kCols>), raise(k3_pass1<float2, L, FftCfg<float2>::kCols>), raise(k4_pass2_store<double2, L>),       \
               raise(k4_pass2_ip<double2, double, AccD, L, false>), raise(k4_pass2_ip<float2, float, AccF, L, false>), \
               raise(k4_pass2_ip<double2, double, AccD, L, true>), raise(k4_pass2_ip<float2, float, AccF, L, true>)
   P2S(5); P2S(6); P2S(7);
@@ -1312,6 +1382,7 @@ void fft_set_smem_limits() {
 #define P3(L) raise(k4_pass2_ip_r8<L, false>), raise(k4_pass2_ip_r8<L, true>)
   P3(8); P3(9); P3(10); P3(11); P3(12);
 #undef P3
+  return fxfft::upload_tables();
 }
 
 }  // namespace emri

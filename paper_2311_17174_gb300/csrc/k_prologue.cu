@@ -270,9 +270,9 @@ __global__ void k0_delay_table(const WalkerC* __restrict__ wc, int n1, int n2, C
       vx = t;
     }
     // columns of 256 rows or more: the fixed-point pass 2 takes the factors as
-    // (cos.h, cos.l, sin.h, sin.l) in Q62
+    // (cos.h, cos.l, sin.h, sin.l), Q62 in balanced halves
     if (!row && n1 >= 256) {
-      const fx::Op a = fx::op(llrint(vx * 0x1p62)), b = fx::op(llrint(vy * 0x1p62));
+      const fx::Op a = fx::bal(llrint(vx * 0x1p62)), b = fx::bal(llrint(vy * 0x1p62));
       *reinterpret_cast<int4*>(dst) = make_int4(a.h, a.l, b.h, b.l);
     } else {
       *dst = make_double2(vx, vy);
