@@ -1057,12 +1057,16 @@ __global__ void __launch_bounds__(kTile, 3) k2_wave_f64(const Knot* __restrict__
 // 20; 114 paired with the quadratics evaluated per sample, 35.0 -> 33.8 ms for
 // 1024 walkers x 2^21).  Four CTAs per SM at 64 registers (three at 80: the
 // same).
+// The set-up's barriers leave the other warps of a CTA idle: with four warps a
+// CTA instead of eight 33.8 -> 33.3 ms (333 walkers x 2^18: 0.894 -> 0.869 ms);
+// a call that does not fill the GPU keeps eight (8 walkers x 2^16: 16 against
+// 22 us).
 //
 // exact_f: exact patterns per sample (long sample intervals), dphib: the
 // LISA orbital phase step per sample [cycles] for them.  No FP64 instruction
 // runs per thread: e0 is tested once per CTA.
-template <int kSegM>
-__global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
+template <int kSegM, int kMixThreads>
+__global__ void __launch_bounds__(kMixThreads, 1024 / kMixThreads) k2_wave_mixed(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
                                                           int64_t n, int exact_f, float dphib, int ks, int n_max,
                                                           float2* __restrict__ z, int unit_scale,
                                                           const float* __restrict__ bc, const float* __restrict__ ifact,
@@ -1071,7 +1075,7 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
   __shared__ IvM iv[kSegM / 64];
   __shared__ float bnode[3 * 32 * 3];
   __shared__ __align__(16) float bq[32 * kQuadStride];
-  __shared__ BlkAmp amps[kTile / 32][32];
+  __shared__ BlkAmp amps[kMixThreads / 32][32];
   __shared__ float fn[kTiles][4][4];   // the four patterns at the fit nodes of each tile
   __shared__ __align__(16) float2 fq[kTiles][4][4];   // their cubics in (t mod 256) / 256, each coefficient twice
   __shared__ float cs0[kTiles][2];     // cos, sin phibar at each tile's start
@@ -1089,12 +1093,12 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
   const int64_t jplunge = C.j_plunge;
   z += (int64_t)wk * n + j0;
   if (jplunge <= j0) {   // nothing left of the inspiral
-    for (int r = t; r < kSegM; r += kTile) z[r] = make_float2(0.f, 0.f);
+    for (int r = t; r < kSegM; r += kMixThreads) z[r] = make_float2(0.f, 0.f);
     return;
   }
   if (t < ni) iv[t] = ivs[(int64_t)wk * nk + kfirst + t];
-  if (t >= 128 && t < 128 + 4 * kTiles) {   // node q of tile tt
-    const int i = t - 128, tt = i / 4, q = i % 4;
+  if (t >= kMixThreads - 4 * kTiles) {   // node q of tile tt
+    const int i = t - (kMixThreads - 4 * kTiles), tt = i / 4, q = i % 4;
     const double* L = lisa + (blockIdx.x * kTiles + tt) * 8 + 2 * q;
     const float cb = (float)L[0], sb = (float)L[1];
     antenna_fixed<float>(C.gf, cb, sb, scale, fn[tt][q]);
@@ -1103,7 +1107,7 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
       cs0[tt][1] = sb;
     }
   }
-  if (t == 224) {
+  if (t == 0) {
     const Geo<float>& G = C.gf;
     g = G;
     gk[0] = make_float4(G.pe1, G.pe1, -G.pe2, -G.pe2);
@@ -1114,8 +1118,8 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
     cheb_s = C.e0 < 0.5;
   }
   __syncthreads();
-  if (t >= 128 && t < 128 + 4 * kTiles) {   // pattern q of tile tt
-    const int i = t - 128, tt = i / 4, q = i % 4;
+  if (t >= kMixThreads - 4 * kTiles) {   // pattern q of tile tt
+    const int i = t - (kMixThreads - 4 * kTiles), tt = i / 4, q = i % 4;
     float cf[4];
     fit_cubic4<float>(fn[tt][0][q], fn[tt][1][q], fn[tt][2][q], fn[tt][3][q], cf);
 #pragma unroll
@@ -1162,7 +1166,7 @@ __global__ void __launch_bounds__(kTile, 4) k2_wave_mixed(const Knot* __restrict
     __sincosf(f.y, &sn.y, &cs.y);
   };
 #pragma unroll 1
-  for (int rb = wq * kBlk; rb < kSegM; rb += kTile / 32 * kBlk) {
+  for (int rb = wq * kBlk; rb < kSegM; rb += kMixThreads / 32 * kBlk) {
     if (rb >= jv) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) z[rb + 32 * i + lane] = make_float2(0.f, 0.f);
@@ -1272,11 +1276,14 @@ void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double 
       float2* zz = (float2*)z + (int64_t)w0 * n;
       const IvM* iv = (const IvM*)ivs + (int64_t)w0 * nk;
       const int us = unit_scale ? 1 : 0;
-#define EMRI_WAVE_MIXED(SEG) \
-  k2_wave_mixed<SEG><<<grid, kTile, 0, s>>>(kn, wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
-      if (seg == 4096) EMRI_WAVE_MIXED(4096);
-      else if (seg == 2048) EMRI_WAVE_MIXED(2048);
-      else EMRI_WAVE_MIXED(1024);
+#define EMRI_WAVE_MIXED(SEG, TH) \
+  k2_wave_mixed<SEG, TH><<<grid, TH, 0, s>>>(kn, wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
+      // four warps a CTA where all CTA slots (eight an SM) are taken, eight
+      // where they are not; a sample's result is the same
+      if (seg == 4096 && n / seg * ww >= 8 * 152) EMRI_WAVE_MIXED(4096, 128);
+      else if (seg == 4096) EMRI_WAVE_MIXED(4096, 256);
+      else if (seg == 2048) EMRI_WAVE_MIXED(2048, 256);
+      else EMRI_WAVE_MIXED(1024, 256);
 #undef EMRI_WAVE_MIXED
     }
   }
