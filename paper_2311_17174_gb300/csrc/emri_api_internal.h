@@ -134,6 +134,10 @@ struct emri_ctx {
   int pipe[2] = {1, 0};
   cudaStream_t pstream[2] = {nullptr, nullptr};
   std::vector<cudaEvent_t> pev;
+  // side stream of a likelihood call's delay constants and tables, and the
+  // events of its fork and join (used under mu)
+  cudaStream_t side = nullptr;
+  cudaEvent_t side_ev[2] = {nullptr, nullptr};
 };
 
 struct emri_dataset {
@@ -160,10 +164,13 @@ size_t loglike_layout(const FftPlan& p, const OptsN& o, int w, int wave, Carve* 
 int pick_wave(emri_ctx* ctx, const FftPlan& p, const OptsN& o, int w);
 int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int64_t ld, int w, const OptsN& o,
                 int wave, const LoglikeBufs& b, double* lnl, double* dh, double* hh, uint32_t* status,
-                cudaStream_t s, int64_t* launches, const FdW* fd = nullptr, int pipe = 1);
+                cudaStream_t s, int64_t* launches, const FdW* fd = nullptr, int pipe = 1, bool side = false);
 // walker groups for a likelihood call on stream s: the context's setting for
 // the precision (0: by the call's size), 1 while s is being captured
 int pipe_groups(emri_ctx* ctx, const OptsN& o, cudaStream_t s);
+// whether such a call may put its delay tables on the context's side stream:
+// not while s is being captured, and only for callers that hold ctx->mu
+bool may_side(cudaStream_t s);
 int ctx_plan_wave(emri_ctx* ctx, int64_t n, const OptsN& o);
 int ctx_plan_ks(emri_ctx* ctx, int64_t n, const OptsN& o);
 void serve_shutdown(emri_ctx* ctx);

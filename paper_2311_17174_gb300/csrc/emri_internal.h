@@ -61,8 +61,11 @@ int upload_bessel_tables(const BesselTab& t);
 // the FP64 waveform kernel's exp(2 pi i k/512) table on the current device; 0 on success
 int upload_exp512();
 
+// the walkers' constants: all of them, all but the delay's (which only the
+// delay tables and pass 2 read), or the delay's
+enum class ProPart { kAll, kNoDelay, kDelay };
 void launch_prologue(const double* theta, int64_t ld, int w, int64_t n, double dt, const OptsN& o,
-                     const double* gl, WalkerC* out, cudaStream_t s);
+                     const double* gl, WalkerC* out, cudaStream_t s, ProPart part = ProPart::kAll);
 // (FP64 tab with n1 >= 256: (cos.h, cos.l, sin.h, sin.l) in Q62, balanced halves (fx64.cuh), four ints)
 // tab[w][n1] = exp(-2 pi i frac(n2 k1 r)), rtab[w][n2] = exp(-2 pi i frac(k2 r))
 void launch_delay_table(const WalkerC* wc, int w, int n1, int n2, bool fp32, void* tab, void* rtab, cudaStream_t s);

@@ -176,7 +176,7 @@ int stretch_run(emri_ctx* ctx, const emri_dataset* ds, double* theta, double* ln
       nl += 1;
     }
     rc = run_loglike(ctx, ds, y, m, m, o, std::min(wave, m), b, lly, nullptr, nullptr, sty, s, &nl, fdw,
-                     pipe_groups(ctx, o, s));
+                     pipe_groups(ctx, o, s), may_side(s));
     k_stretch_accept<<<gb, tb, 0, s>>>(theta, lnp, w, a0, m, y, zs, lly, sty, u, sa, accepted);
     nl += 2;
   }

@@ -66,9 +66,9 @@ constexpr int kProWalkers = 8;   // walkers per CTA (four lanes each in the quad
 __global__ void __launch_bounds__(128) k0_prologue(const double* __restrict__ theta, int64_t ld, int w, int64_t n,
                                                    double dt, int mode, double n_xi, double omega_m, double h0,
                                                    ProConst K, const double* __restrict__ gl,
-                                                   WalkerC* __restrict__ out) {
+                                                   WalkerC* __restrict__ out, int role0) {
   __shared__ int bad_dgw[kProWalkers];
-  const int role = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int role = role0 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int slot = role == 2 ? lane >> 2 : lane;        // the quadrature takes four lanes per walker
   const int i = blockIdx.x * kProWalkers + slot;
   const bool mine = slot < kProWalkers && i < w;
@@ -162,6 +162,9 @@ __global__ void __launch_bounds__(128) k0_prologue(const double* __restrict__ th
     f.spS = (float)g.spS; f.sqS = (float)g.sqS;
     f.sin_ths = (float)sts; f.cos_ths = (float)cts; f.sin_phs = (float)sps; f.cos_phs = (float)cps;
     f.amp_scale = (float)g.amp_scale;
+    c.pad[0] = c.pad[1] = c.pad[2] = 0.0;
+    c.j_plunge = n;
+    c.pad_u = 0;
   } else if (role == 2) {
     // d_L(z) = (1+z)(c/H0) int_0^z dz'/E(z'), E = sqrt(Om (1+z)^3 + 1 - Om);
     // lane sub of a walker's four takes the nodes q = sub mod 4
@@ -206,11 +209,8 @@ __global__ void __launch_bounds__(128) k0_prologue(const double* __restrict__ th
     c.r_lo = r_lo;
     c.cn_re = cn;
     c.cn_im = sn;
-    c.pad[0] = c.pad[1] = c.pad[2] = 0.0;
     c.cnf[0] = (float)cn;
     c.cnf[1] = (float)sn;
-    c.j_plunge = n;
-    c.pad_u = 0;
   }
   __syncthreads();
   if (role == 0 && mine) out[i].status = st | (bad_dgw[slot] ? (uint32_t)ST_BADPARAM : 0u);
@@ -293,10 +293,11 @@ __global__ void k0_export(const WalkerC* __restrict__ wc, int w, double* __restr
 }
 
 void launch_prologue(const double* theta, int64_t ld, int w, int64_t n, double dt, const OptsN& o,
-                     const double* gl, WalkerC* out, cudaStream_t s) {
+                     const double* gl, WalkerC* out, cudaStream_t s, ProPart part) {
   if (w <= 0) return;
-  k0_prologue<<<(w + kProWalkers - 1) / kProWalkers, 128, 0, s>>>(theta, ld, w, n, dt, o.mode, o.n_xi, o.omega_m,
-                                                                  o.h0, pro_const(o.omega_m, o.h0), gl, out);
+  const int role0 = part == ProPart::kDelay ? 3 : 0, roles = part == ProPart::kAll ? 4 : part == ProPart::kDelay ? 1 : 3;
+  k0_prologue<<<(w + kProWalkers - 1) / kProWalkers, 32 * roles, 0, s>>>(
+      theta, ld, w, n, dt, o.mode, o.n_xi, o.omega_m, o.h0, pro_const(o.omega_m, o.h0), gl, out, role0);
 }
 
 void launch_delay_table(const WalkerC* wc, int w, int n1, int n2, bool fp32, void* tab, void* rtab, cudaStream_t s) {

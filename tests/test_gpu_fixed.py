@@ -102,3 +102,49 @@ def test_waveform_knot_spacings(ctx, ks, n_max):
         tol = 1e-9 * max(1.0, (ks / 128) ** 4)
         assert rel(got[k], ref) <= tol, (k, rel(got[k], ref))
         assert np.abs(got[k] - ref).max() <= tol * np.abs(ref).max(), k
+
+
+def test_side_stream_order(ctx):
+    """The delay tables run on the context's side stream: calls in a row on
+    two user streams, with other walkers each, give the same bits as the same
+    calls one at a time, and so does a captured call (which keeps one stream;
+    a context captures on the stream of its last call)."""
+    from paper_2311_17174_gb300 import emri as E
+    n, dt, w = 1 << 13, 15.0, 5
+    psd = I.psd_bc04(n, dt)
+    noise = I.noise_spectrum(9, psd, n, dt)
+    ds = ctx.dataset(E.grid(n, dt), noise, psd, 1e-4, 1.0 / (2 * dt))
+    th = [torch.tensor(I.draw_sources(60 + k, w, n).T.copy(), device="cuda:0") for k in range(6)]
+    for prec in (E.FP64, E.MIXED):
+        o = E.opts(precision=prec, n_max=6)
+        alone = []
+        for t in th:
+            out = torch.zeros(w, dtype=torch.float64, device="cuda:0")
+            ctx.loglike_batch(ds, t, o, out)
+            torch.cuda.synchronize()
+            alone.append(out.cpu().numpy())
+        streams = [torch.cuda.Stream() for _ in range(2)]
+        outs = [torch.zeros(w, dtype=torch.float64, device="cuda:0") for _ in th]
+        torch.cuda.synchronize()
+        for k, t in enumerate(th):
+            ctx.loglike_batch(ds, t, o, outs[k], stream=streams[k % 2])
+        torch.cuda.synchronize()
+        for k in range(len(th)):
+            np.testing.assert_array_equal(outs[k].cpu().numpy(), alone[k])
+        c2 = E.Context(0)
+        ds2 = c2.dataset(E.grid(n, dt), noise, psd, 1e-4, 1.0 / (2 * dt))
+        out = torch.zeros(w, dtype=torch.float64, device="cuda:0")
+        torch.cuda.synchronize()
+        c2.loglike_batch(ds2, th[3], o, out, stream=streams[0])
+        torch.cuda.synchronize()
+        out.zero_()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=streams[0]):
+            c2.loglike_batch(ds2, th[3], o, out, stream=streams[0])
+        g.replay()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(out.cpu().numpy(), alone[3])
+        ds2.close()
+        c2.close()
+    ds.close()
