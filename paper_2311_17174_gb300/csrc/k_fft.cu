@@ -832,11 +832,13 @@ struct AccF {
 struct U128 {
   unsigned long long hi, lo;
 };
-__device__ __forceinline__ U128 mul128_small(U128 a, unsigned long long k) {
-  U128 r;
-  r.lo = a.lo * k;
-  r.hi = a.hi * k + __umul64hi(a.lo, k);
-  return r;
+// a k: four 32 x 32-bit multiply-adds (the bin index has 22 bits; a 64-bit k
+// took ~18 instructions)
+__device__ __forceinline__ U128 mul128_small(U128 a, uint32_t k) {
+  const fx::u64 r0 = fx::wideu((uint32_t)a.lo, k, 0), r1 = fx::wideu((uint32_t)(a.lo >> 32), k, r0 >> 32);
+  const fx::u64 r2 = fx::wideu((uint32_t)a.hi, k, r1 >> 32);
+  const uint32_t r3 = (uint32_t)(a.hi >> 32) * k + (uint32_t)(r2 >> 32);
+  return U128{((fx::u64)r3 << 32) | (uint32_t)r2, (r1 << 32) | (uint32_t)r0};
 }
 __device__ __forceinline__ U128 add128(U128 a, U128 b) {
   U128 r;
@@ -870,28 +872,51 @@ __device__ __forceinline__ void phase_factor(long long top, float& c, float& s) 
 __device__ __forceinline__ double fd_exp(double x) { return exp(x); }
 __device__ __forceinline__ float fd_exp(float x) { return __expf(x); }
 
-// Frequency-dependent factor of bin |k_s| = a: amplitude A (returned) and
-// the phase factor (c, s) = exp(-2 pi i sgn(k_s) sum beta_m a^(m+1)).
+// A walker's propagation record in the kernel's type, in shared memory: the
+// conversions (FP64 pipe) once per CTA.  With it and the four-instruction
+// mul128_small: 333 walkers x 2^18 mixed, pass 2 0.737 -> 0.529 ms.
 template <typename T>
-__device__ __forceinline__ T fd_factor(const FdW& f, unsigned long long a, bool neg, T& c, T& s) {
-  T A = T(1);
-  if (f.qm > 0) {
-    const T x = (T)a * (T)f.xs;
-    T am = (T)f.a[f.qm - 1];
-    for (int m = f.qm - 2; m >= 0; --m) am = am * x + (T)f.a[m];
-    A = fd_exp((T)f.nlz_half * am * x);
+struct FdRec {
+  T nlz_half, xs, a[3];
+  U128 b[3];
+  int qm, qt;
+  __device__ void set(const FdW& f) {
+    nlz_half = (T)f.nlz_half;
+    xs = (T)f.xs;
+    qm = f.qm;
+    qt = f.qt;
+    for (int m = 0; m < 3; ++m) {
+      a[m] = (T)f.a[m];
+      b[m] = U128{f.bhi[m], f.blo[m]};
+    }
   }
-  if (f.qt > 0) {
-    U128 acc{f.bhi[f.qt - 1], f.blo[f.qt - 1]};
-    for (int m = f.qt - 2; m >= 0; --m) acc = add128(mul128_small(acc, a), U128{f.bhi[m], f.blo[m]});
-    acc = mul128_small(mul128_small(acc, a), a);
-    if (neg) acc = neg128(acc);
-    phase_factor((long long)acc.hi, c, s);
-  } else {
-    c = T(1);
-    s = T(0);
-  }
-  return A;
+};
+
+// Frequency-dependent factor of bin |k_s| = a: the amplitude A ...
+template <typename T>
+__device__ __forceinline__ T fd_amp(const FdRec<T>& f, uint32_t a) {
+  if (f.qm <= 0) return T(1);
+  const T x = (T)a * f.xs;
+  T am = f.a[f.qm - 1];
+  for (int m = f.qm - 2; m >= 0; --m) am = am * x + f.a[m];
+  return fd_exp(f.nlz_half * am * x);
+}
+// ... and sgn(k_s) sum beta_m a^(m+1), the phase in cycles mod 1 (top 64 bits;
+// the factor is exp(-2 pi i phase))
+template <typename T>
+__device__ __forceinline__ unsigned long long fd_phase(const FdRec<T>& f, uint32_t a, bool neg) {
+  if (f.qt <= 0) return 0;
+  U128 acc = f.b[f.qt - 1];
+  for (int m = f.qt - 2; m >= 0; --m) acc = add128(mul128_small(acc, a), f.b[m]);
+  acc = mul128_small(mul128_small(acc, a), a);
+  return neg ? neg128(acc).hi : acc.hi;
+}
+template <typename T>
+__device__ __forceinline__ T fd_factor(const FdRec<T>& f, uint32_t a, bool neg, T& c, T& s) {
+  c = T(1);
+  s = T(0);
+  if (f.qt > 0) phase_factor((long long)fd_phase(f, a, neg), c, s);
+  return fd_amp(f, a);
 }
 
 // Shared memory of one pass-2 row: the row itself, then (when they fit in
@@ -945,8 +970,11 @@ __global__ void __launch_bounds__(kPass2Threads, sizeof(C2) == 8 ? 4 : 2)
   // frequencies; the table carries it for k1 > N1/2), and the row factor a
   // is common to the row: <d|h> collects Z = sum g ts H and takes Re(a Z).
   T zr = T(0), zi = T(0), shh = T(0);
-  FdW fd;
-  if (FD) fd = fdw[wk];
+  __shared__ FdRec<T> fd;
+  if (FD) {
+    if (threadIdx.x == 0) fd.set(fdw[wk]);
+    __syncthreads();
+  }
   for (int k1 = threadIdx.x; k1 < N1; k1 += kPass2Threads) {
     const C2 H = buf[k1];
     const T wv = SM::kPrefetch ? (T)ws[k1] : (T)wperm[base + k1];
@@ -957,7 +985,7 @@ __global__ void __launch_bounds__(kPass2Threads, sizeof(C2) == 8 ? 4 : 2)
     if (FD) {
       const bool neg = 2 * k1 > N1 || (2 * k1 == N1 && k2 > 0);
       const long long kk = (long long)k2 + (long long)n2 * k1;
-      const unsigned long long ak = (unsigned long long)(neg ? n - kk : kk);
+      const uint32_t ak = (uint32_t)(neg ? n - kk : kk);
       T c, sn;
       const T A = fd_factor<T>(fd, ak, neg, c, sn);
       P = cmul(P, CT<C2>::make(A * c, A * sn));
@@ -1000,8 +1028,10 @@ __global__ void __launch_bounds__((1 << LG) / 8)
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* xb = reinterpret_cast<float2*>(smraw);   // stage exchange, padded
   __shared__ AccF red[T / 32];
+  __shared__ FdRec<float> fd;
   const int t = threadIdx.x;
   const int k2 = blockIdx.x, wk = blockIdx.y;
+  if (FD && t == 0) fd.set(fdw[wk]);   // (read after the stages' barriers)
   const int64_t base = (int64_t)k2 * N1;
   // the inner product's operands, read where they are used (the row's
   // dataset entries from L2, the walker's delay factors from L1/L2): shared
@@ -1022,8 +1052,6 @@ __global__ void __launch_bounds__((1 << LG) / 8)
   r8::last_stage<LG>(v, tt, t);
   // the thread's bins k1 = t + q T in plain FP32, then the compensated tree
   float zr = 0.f, zi = 0.f, shh = 0.f;
-  FdW fd;
-  if (FD) fd = fdw[wk];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int k1 = t + q * T;
@@ -1038,7 +1066,7 @@ __global__ void __launch_bounds__((1 << LG) / 8)
     if (FD) {
       const bool neg = q > 4 || (q == 4 && t > 0) || (q == 4 && t == 0 && k2 > 0);
       const long long kk = (long long)k2 + (long long)n2 * k1;
-      const unsigned long long ak = (unsigned long long)(neg ? n - kk : kk);
+      const uint32_t ak = (uint32_t)(neg ? n - kk : kk);
       float c, sn;
       const float A = fd_factor<float>(fd, ak, neg, c, sn);
       P = cmul(P, make_float2(A * c, A * sn));
