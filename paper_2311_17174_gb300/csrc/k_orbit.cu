@@ -26,8 +26,9 @@
 //   k1e_knots    the knots every K_s samples, read off the segment's
 //                polynomial (integral weights at the knot positions), one
 //                knot per lane over the whole GPU;
-//   k1f_tail     walkers whose orbit reaches the LSO, turns non-finite or
-//                does not settle: the rest of the orbit from the first such
+//   k1f_tail     walkers whose orbit reaches the LSO: the plunge sample, from
+//                the knots around it; walkers whose orbit turns non-finite
+//                or does not settle: the rest of the orbit from the first such
 //                segment, in sequence (Picard sweeps, then knot-step RK4).
 // The bound is the FP64 pipe when many walkers fill the GPU and the latency
 // of the launch chain when few do.  One warp per walker doing all of it in
@@ -50,7 +51,7 @@
 // phase has no rounding drift.  Each knot stores the state and its rates;
 // the Doppler delay nu (R/c) sin(theta_S) cos(phibar - phi_S) is folded into
 // the stored phase, and the sample at which nu reaches nu_LSO(e) (paper
-// Sec. 3) is located by re-integrating the crossing interval at step dt.
+// Sec. 3) is located inside the crossing knot interval.
 #include "emri_common.cuh"
 #include "emri_internal.h"
 

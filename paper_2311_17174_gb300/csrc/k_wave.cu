@@ -1,21 +1,21 @@
 // k_wave.cu -- steps S2-S4: dense orbit, LISA response and the
-// Peters-Mathews harmonic sum of Eq. (2), one CTA per 256-sample tile (FP64)
-// or per 1024-sample segment (mixed).
+// Peters-Mathews harmonic sum of Eq. (2), one CTA per one or four 1024-sample
+// segments (FP64) or per segment of up to 4096 samples (mixed).
 //
-// Per tile (set-up, a few threads):
+// Per segment (set-up):
 //  * the cubic Hermite interpolant of every orbit quantity over each knot
-//    interval the tile touches (values and rates at both knots);
-//  * the Bessel amplitudes of every harmonic at the tile's start, middle and
-//    end, fitted by a quadratic in time.  The amplitudes depend on time only
-//    through e(t), which moves by ~1e-4 relative per tile, so the quadratic
-//    is exact to ~1e-11 and the per-sample cost of a harmonic drops from a
-//    Bessel evaluation to a few FMAs;
+//    interval (values and rates at both knots);
+//  * the Bessel amplitudes of every harmonic at the segment's start, middle
+//    and end, fitted by a quadratic in time.  The amplitudes depend on time
+//    only through e(t), which moves by ~1e-4 relative per 256 samples, so the
+//    quadratic is exact to ~1e-14 over 1024 and the per-sample cost of a
+//    harmonic drops from a Bessel evaluation to a few FMAs;
 //  * the four antenna patterns in a fixed sky polarisation basis at four
-//    nodes, fitted by a cubic in time (they depend on time only through the
-//    LISA orbital phase, a one-year period).
-// Per sample (one thread each; four per thread in the mixed kernel):
+//    nodes of each 256-sample tile, fitted by a cubic in time (they depend on
+//    time only through the LISA orbital phase, a one-year period).
+// Per sample:
 //  * phases Phi_D (Doppler folded in), 2 gamma~ and alpha from the Hermite
-//    polynomials, reduced modulo one cycle, and their sin/cos;
+//    polynomials, modulo one cycle, and their sin/cos;
 //  * the harmonic sum written as three running sums
 //      C = sum_n n pa_n cos(n Phi), S = sum_n n sqrt(1-e^2) pb_n sin(n Phi),
 //      R = sum_n 2 pc_n cos(n Phi),
@@ -26,9 +26,10 @@
 //    cos alpha, sin alpha), times the fitted patterns -- identical to the
 //    psi / beta form of the Barack-Cutler response, without either angle;
 //  * z = h_I + i h_II.
-// FP64 variant: everything in double.  Mixed variant: the three phases are
-// evaluated in 64-bit fixed point (linear term) plus an FP32 correction, so
-// no FP64 instruction runs per sample; the rest is FP32.
+// FP64 variant: phases, sums and response in 64-bit fixed point, the slowly
+// varying factors in double (all of it in double outside the fixed-point
+// ranges).  Mixed variant: the phases in 64-bit fixed point (linear term) plus
+// an FP32 correction, the rest in FP32; no FP64 instruction runs per sample.
 #include <vector>
 #include "emri_common.cuh"
 #include "fx64.cuh"
@@ -1052,11 +1053,12 @@ __global__ void __launch_bounds__(kTile, 3) k2_wave_f64(const Knot* __restrict__
 // of the segment's, is below FP32 resolution except close to a plunge
 // (`curved`), so a harmonic takes 8 paired FMAs per pair of samples instead
 // of 11 and three 16-byte loads instead of five; the samples of a pair lie 32
-// apart in one knot interval, and share its record, the pattern cubics and the phase's 64-bit product.  Bound
-// by the FMA pipe (99 paired and ~170 other instructions a sample at n_max =
-// 20; 114 paired with the quadratics evaluated per sample, 35.0 -> 33.8 ms for
-// 1024 walkers x 2^21).  Four CTAs per SM at 64 registers (three at 80: the
-// same).
+// apart in one knot interval, and share its record, the pattern cubics and the
+// phase's 64-bit product.  Bound by instruction issue: 99 paired instructions, two slots each, and ~170 others
+// a sample at n_max = 20 (114 paired with the quadratics evaluated per sample,
+// 35.0 -> 33.8 ms for 1024 walkers x 2^21).  kOneIv (K_s >= 128): the block's
+// four samples share one interval record; with it and 24 warps per SM at 80
+// registers 33.2 -> 32.8 ms (at 64 registers it spills: 34.1 ms).
 // The set-up's barriers leave the other warps of a CTA idle: with four warps a
 // CTA instead of eight 33.8 -> 33.3 ms (333 walkers x 2^18: 0.894 -> 0.869 ms);
 // a call that does not fill the GPU keeps eight (8 walkers x 2^16: 16 against
@@ -1065,8 +1067,8 @@ __global__ void __launch_bounds__(kTile, 3) k2_wave_f64(const Knot* __restrict__
 // exact_f: exact patterns per sample (long sample intervals), dphib: the
 // LISA orbital phase step per sample [cycles] for them.  No FP64 instruction
 // runs per thread: e0 is tested once per CTA.
-template <int kSegM, int kMixThreads>
-__global__ void __launch_bounds__(kMixThreads, 1024 / kMixThreads) k2_wave_mixed(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
+template <int kSegM, int kMixThreads, bool kOneIv>
+__global__ void __launch_bounds__(kMixThreads, 768 / kMixThreads) k2_wave_mixed(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
                                                           int64_t n, int exact_f, float dphib, int ks, int n_max,
                                                           float2* __restrict__ z, int unit_scale,
                                                           const float* __restrict__ bc, const float* __restrict__ ifact,
@@ -1198,7 +1200,7 @@ __global__ void __launch_bounds__(kMixThreads, 1024 / kMixThreads) k2_wave_mixed
     float2 c1[2], s1[2], Cs[2], Ss[2], Rs[2];
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-      const int ki = (rb + 64 * p) >> lks, tau = rb + 64 * p + lane - (ki << lks);
+      const int ki = (kOneIv ? rb : rb + 64 * p) >> lks, tau = rb + 64 * p + lane - (ki << lks);
       const float2 s = make_float2((float)tau * inv_ks, (float)(tau + 32) * inv_ks);
       const IvM& v = iv[ki];
       sincos2(v.ph_base, v.ph_inc, v.ph_c, tau, s, c1[p], s1[p]);
@@ -1208,7 +1210,7 @@ __global__ void __launch_bounds__(kMixThreads, 1024 / kMixThreads) k2_wave_mixed
     const int tt = rb / kTile;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-      const int ki = (rb + 64 * p) >> lks, tau = rb + 64 * p + lane - (ki << lks);
+      const int ki = (kOneIv ? rb : rb + 64 * p) >> lks, tau = rb + 64 * p + lane - (ki << lks);
       const float2 s = make_float2((float)tau * inv_ks, (float)(tau + 32) * inv_ks);
       const IvM& v = iv[ki];
       float2 c2g, s2g, ca, sa, F[4], hI, hII;
@@ -1276,11 +1278,12 @@ void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double 
       float2* zz = (float2*)z + (int64_t)w0 * n;
       const IvM* iv = (const IvM*)ivs + (int64_t)w0 * nk;
       const int us = unit_scale ? 1 : 0;
-#define EMRI_WAVE_MIXED(SEG, TH) \
-  k2_wave_mixed<SEG, TH><<<grid, TH, 0, s>>>(kn, wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
-      // four warps a CTA where all CTA slots (eight an SM) are taken, eight
+#define EMRI_WAVE_MIXED(SEG, TH)                                                                                       \
+  (o.ks >= kBlk ? k2_wave_mixed<SEG, TH, true> : k2_wave_mixed<SEG, TH, false>)<<<grid, TH, 0, s>>>(                   \
+      kn, wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
+      // four warps a CTA where all CTA slots (six an SM) are taken, eight
       // where they are not; a sample's result is the same
-      if (seg == 4096 && n / seg * ww >= 8 * 152) EMRI_WAVE_MIXED(4096, 128);
+      if (seg == 4096 && n / seg * ww >= 6 * 152) EMRI_WAVE_MIXED(4096, 128);
       else if (seg == 4096) EMRI_WAVE_MIXED(4096, 256);
       else if (seg == 2048) EMRI_WAVE_MIXED(2048, 256);
       else EMRI_WAVE_MIXED(1024, 256);
