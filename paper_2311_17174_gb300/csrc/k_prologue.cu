@@ -214,6 +214,16 @@ __global__ void __launch_bounds__(128) k0_prologue(const double* __restrict__ th
   }
   __syncthreads();
   if (role == 0 && mine) out[i].status = st | (bad_dgw[slot] ? (uint32_t)ST_BADPARAM : 0u);
+  // a walker whose d_GW is not positive has no delay either.  (The delay's own
+  // launch does not know d_GW; nothing reads that walker's delay there, its
+  // waveform is zero.)
+  if (role == 3 && role0 == 0 && mine && bad_dgw[slot]) {
+    WalkerC& c = out[i];
+    c.dt_gw = c.r_hi = c.r_lo = c.cn_im = 0.0;
+    c.cn_re = 1.0;
+    c.cnf[0] = 1.f;
+    c.cnf[1] = 0.f;
+  }
 }
 
 // Per-walker delay tables for the factorisation
