@@ -15,8 +15,9 @@
 //   k1b_eval     one warp per segment, three (rarely four) times: the FP64
 //                rates at the nodes and the FP64 residual of the collocation
 //                equations; the linearised correction is solved in FP32 (its
-//                relative error, ~1e-4, is the contraction per evaluation:
-//                1e-6 -> 5e-11 -> 1e-15 -> below rounding), with the
+//                relative error, ~1e-4 to 1e-3, is the contraction per
+//                evaluation: 1e-6 -> 1e-10 -> 1e-14 -> below rounding;
+//                orbit_rule.cuh measures it and decides), with the
 //                corrections of the segments' start values carried across
 //                segments by the product of their 2x2 propagators;
 //   k1c_final    the last correction, then all five rates at the nodes and
@@ -54,6 +55,7 @@
 // Sec. 3) is located inside the crossing knot interval.
 #include "emri_common.cuh"
 #include "emri_internal.h"
+#include "orbit_rule.cuh"
 
 namespace emri {
 
@@ -273,11 +275,6 @@ __device__ __forceinline__ OrbWork orb_work(char* base, int64_t wk, int64_t ns) 
   return o;
 }
 
-// A correction above kUpdateAgain at the third evaluation asks for a fourth
-// one; the last correction has to stay below kUpdateDone (the error left is
-// about 1e-4 of it).
-constexpr float kUpdateAgain = 1e-9f, kUpdateDone = 1e-12f;
-
 // Walker's start state in integration order: the prologue's values, and in
 // backward mode (paper Sec. 3: initial conditions at the LSO, integrated back
 // in time; the LSO state sits at the last sample t0 + (n-1) dt) one RK4 step
@@ -487,7 +484,7 @@ __device__ __forceinline__ float2 solve_linear(float2 r, const float4& J, float 
 // the previous values plus their correction), the FP64 rates, the residual of
 // the collocation equations and the segment's own FP32 correction.  kIt = 0
 // also builds the node Jacobians and the propagators; kIt = 3 runs only for
-// walkers whose third correction was above kUpdateAgain.  About 145 FP64
+// walkers that need it (orbit_again).  About 145 FP64
 // instructions per lane and evaluation (70 for the rates, 64 for the node
 // sums), which bound it.
 template <int kIt>
@@ -504,7 +501,7 @@ __global__ void __launch_bounds__(32 * kEvalWarps) k1b_eval(const WalkerC* __res
   const OrbWork o = orb_work(orb, wk, ns);
   const int good = o.flag[0];
   if ((int)(blockIdx.x * kEvalWarps) >= good) return;
-  if (kIt == 3 && __int_as_float(o.flag[3]) <= kUpdateAgain) return;
+  if (kIt == 3 && !orbit_again(__int_as_float(o.flag[2]), __int_as_float(o.flag[3]))) return;
   for (int t = threadIdx.x; t < 32 * 32; t += blockDim.x) {
     const double q = qn_g[t];
     qn[t] = q;
@@ -593,7 +590,8 @@ __global__ void __launch_bounds__(32 * kEvalWarps) k1b_eval(const WalkerC* __res
   float4 J;
   const float Hf = (float)H;
   if constexpr (kIt == 0) {
-    // central differences of the FP32 rates (relative error ~1e-4)
+    // central differences of the FP32 rates, steps of v/128 and (1 - e^2)/128
+    // (relative error up to 9e-4: v^11)
     const OrbSrcT<float> sf{(float)s.kv, (float)s.ke, (float)s.inv2pim, (float)s.spin, (float)s.cl, pn};
     const float vf = (float)v, ef = (float)e;
     const float hv = vf * 0.0078125f, he = 0.0078125f * (1.f - ef * ef);
@@ -630,8 +628,9 @@ __global__ void __launch_bounds__(32 * kEvalWarps) k1b_eval(const WalkerC* __res
 }
 
 // The last correction, the five rates at the corrected nodes and their
-// integrals over the segment.  A correction above kUpdateDone (or NaN) leaves
-// the walker's remaining segments to k1f_tail.
+// integrals over the segment.  A segment that has not settled leaves the
+// walker's segments from it on to k1f_tail (those before it do not depend on
+// it).
 __global__ void __launch_bounds__(32 * kEvalWarps) k1c_final(const WalkerC* __restrict__ wcs, int64_t n, double dt,
                                                              int ks, int pn, int back,
                                                              const double* __restrict__ qn_g, char* __restrict__ orb) {
@@ -642,10 +641,11 @@ __global__ void __launch_bounds__(32 * kEvalWarps) k1c_final(const WalkerC* __re
   const int i = blockIdx.x * kEvalWarps + wq;
   // [5]: segments the coarse pass reached; [0] is lowered here
   if (i >= o.flag[5]) return;
-  const int p = __int_as_float(o.flag[3]) <= kUpdateAgain ? 0 : 1;
+  const float u1 = __int_as_float(o.flag[2]), u2 = __int_as_float(o.flag[3]);
+  const int p = orbit_again(u1, u2) ? 1 : 0;
   float m;
   const NodeState y = apply_update(o, ns, i, p, lane, m);
-  if (!(m <= kUpdateDone)) {
+  if (!(p ? orbit_settled(u2, __int_as_float(o.flag[4]), m) : orbit_settled(u1, u2, m))) {
     if (lane == 0) atomicMin(&o.flag[0], i);
     return;
   }
@@ -831,10 +831,10 @@ __device__ int plunge_sample(const OrbSrc& s, const OrbState& y0, int ks, double
 // solution does not cover (none for most walkers: then this only writes the
 // status), one warp per walker.  A solved segment that passes the LSO at a
 // knot: the plunge sample (plunge_sample), the knots being there already.
-// Otherwise in sequence: per segment FP64 Picard sweeps,
-// the knots from the segment polynomial, and where the sweeps do not settle
-// or a knot lies past the LSO, knot-step RK4 by lane 0, which also locates the
-// plunge sample.  In backward mode no plunge check applies; an orbit that
+// Otherwise in sequence: per segment FP64 Picard sweeps, the knots from the
+// segment polynomial and the plunge sample as in a solved segment; where the
+// sweeps do not settle, or the plunge moves too fast for that, knot-step RK4
+// by lane 0, which also locates the plunge sample.  In backward mode no plunge check applies; an orbit that
 // turns non-finite gives a zero waveform and ST_NONFINITE.
 __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_t n, double dt,
                                                const double2* __restrict__ cs, int ks,
@@ -869,24 +869,26 @@ __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_
   const int64_t kstart = back ? nk - (int64_t)g0 * K : (int64_t)g0 * K;
   int64_t last = kstart;            // forward: last knot written
   bool done = false;
-  if (!back && g0 < o.flag[0]) {    // solved: the first knot past the LSO is q, counted from the segment's start
-    const int q = o.flag[6] - g0 * K;
-    const double* f5 = reinterpret_cast<const double*>(o.work + (int64_t)g0 * 1280);
-    OrbState ym = y, yq = y;        // knots q - 1 and q
+  // The plunge sample where knot q of the segment that starts at knot kb (state
+  // ys, node rates f5) is its first past the LSO; the knots before it are there
+  // already.  false: not found this way.
+  auto plunge_in = [&](const OrbState& ys, const double* f5, int64_t kb, int q) {
+    OrbState ym = ys, yq = ys;      // knots q - 1 and q
     if (q > 1) knot_state(ym, f5, qk_g + (size_t)(q - 1) * (128 / K) * 32, H);
     knot_state(yq, f5, qk_g + (size_t)q * (128 / K) * 32, H);
     const int d = state_finite(yq) ? plunge_sample(s, ym, ks, dt, lane) : -1;
-    if (d > 0) {
-      last = kstart + q;
-      jp = (last - 1) * ks + d;
-      if (jp < n) st |= ST_PLUNGE;
-      else jp = n;
-      double r[5];
-      ak_rhs_v(s, yq.v_hi, yq.e_hi, r[0], r[1], r[2], r[3], r[4]);
-      if (lane == 0) write_knot(kn, last, yq, r, c, cs, doppler);
-      done = true;
-    }
-  }
+    if (d <= 0) return false;
+    last = kb + q;
+    jp = (last - 1) * ks + d;
+    if (jp < n) st |= ST_PLUNGE;
+    else jp = n;
+    double r[5];
+    ak_rhs_v(s, yq.v_hi, yq.e_hi, r[0], r[1], r[2], r[3], r[4]);
+    if (lane == 0) write_knot(kn, last, yq, r, c, cs, doppler);
+    return true;
+  };
+  if (!back && g0 < o.flag[0])      // solved: the first knot past the LSO, counted from the segment's start
+    done = plunge_in(y, reinterpret_cast<const double*>(o.work + (int64_t)g0 * 1280), kstart, o.flag[6] - g0 * K);
   if (done) {
   } else if (back && !state_finite(y)) {
     fail = true;
@@ -938,6 +940,7 @@ __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_
 #pragma unroll
       for (int q = 0; q < 5; ++q) f[q * 32 + lane] = r[q];
       __syncwarp();
+      int qbad = 0;                  // first knot past the LSO or not finite
       for (int q0 = 1; q0 <= K; q0 += 32) {
         const int q = q0 + lane;
         bool bad = false;
@@ -952,8 +955,16 @@ __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_
             write_knot(kn, k, yk, rk, c, cs, doppler);
           }
         }
-        serial |= __any_sync(0xffffffffu, bad);
+        const unsigned b = __ballot_sync(0xffffffffu, bad);
+        if (b && !qbad) qbad = q0 + __ffs(b) - 1;
         if (K - q0 < 32) y = bcast_state(yk, K - q0);   // the end state, every lane's next start
+      }
+      if (qbad) {
+        if (!back && plunge_in(ys, f, kb, qbad)) {
+          done = true;
+          break;
+        }
+        serial = true;
       }
     }
     if (serial) {
