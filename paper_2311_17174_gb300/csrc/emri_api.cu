@@ -235,9 +235,8 @@ size_t loglike_layout(const FftPlan& p, const OptsN& o, int w, int wave, Carve* 
   LoglikeBufs t;
   t.wc = cv.take<WalkerC>(w);
   t.knots = cv.take<Knot>((size_t)w * (nk + 1));
-  t.orb = cv.take<char>((size_t)w * orbit_bytes(p.n, o.ks));
   t.ivs = cv.take<char>(o.precision ? (size_t)w * nk * kIvMBytes : 0);
-  t.lisa = cv.take<double>(lisa_len(p.n, o.ks));
+  t.lisa = cv.take<double>(lisa_len(p.n));
   t.dtab = cv.take<char>((size_t)w * p.n1 * cs);
   t.rtab = cv.take<char>((size_t)w * p.n2 * cs);
   t.partial = cv.take<double2>((size_t)w * p.n2);
@@ -335,12 +334,11 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
     launch_wave(b.knots + (size_t)j0 * (nk + 1), b.wc + j0, gw, p.n, ds->dt, ds->t0, o, zg, false, ctx->bt,
                 b.lisa, b.ivs + (size_t)j0 * nk * kIvMBytes, st);
   };
-  const size_t ob = orbit_bytes(p.n, o.ks);
-  auto orbit_of = [&](int j0, int gw, cudaStream_t st) {
+  const size_t per = (size_t)p.n * cs;   // bytes of one walker's series
+  auto orbit_of = [&](int j0, int gw, const double2* lk, char* orb, int64_t fit, cudaStream_t st) {
     Knot* kj = b.knots + (size_t)j0 * (nk + 1);
     KTimer t(pf, EMRI_K_ORBIT, st);
-    nl += launch_orbit(b.wc + j0, gw, p.n, ds->dt, lisa_knots(b.lisa, p.n), o, kj, ctx->mcpi, b.orb + (size_t)j0 * ob,
-                       st);
+    nl += launch_orbit(b.wc + j0, gw, p.n, ds->dt, lk, o, kj, ctx->mcpi, orb, fit, st);
     if (f32) {
       launch_intervals_mixed(kj, gw, p.n, o.ks, ds->dt, b.ivs + (size_t)j0 * nk * kIvMBytes, st);
       ++nl;
@@ -376,8 +374,9 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
     }
   }
   if (pipe <= 1) {
-    launch_lisa(p.n, o.ks, ds->t0, ds->dt, b.lisa, s);
-    orbit_of(0, w, s);
+    const OrbScratch os(b.z, (size_t)wave * per, p.n, o.ks);
+    launch_lisa(p.n, o.ks, ds->t0, ds->dt, b.lisa, os.cs, s);
+    orbit_of(0, w, os.cs, os.orb, os.fit, s);
     nl += 3;
     for (int i0 = 0; i0 < w; i0 += wave) {
       const int ww = std::min(wave, w - i0);
@@ -389,23 +388,32 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   } else {
     int rc = pipe_resources(ctx);
     if (rc) return rc;
-    launch_lisa(p.n, o.ks, ds->t0, ds->dt, b.lisa, s);
+    // orbits: the first group's alone, then every other walker's in one
+    // launch that runs beside the first group's waveform (a launch of few
+    // walkers is a chain of nine kernels bound by their latency: one per group
+    // would queue G of them).  Their solver states lie in the series buffer:
+    // the first group's in its own part, which its waveform overwrites once
+    // they are done, the others' in the rest, which the later groups' waveforms
+    // write after every orbit.  Where a wave is a single group, every orbit
+    // comes before the first waveform.
+    const int w1 = std::min(wave, w);
+    const int g0 = (w1 + std::min(pipe, w1) - 1) / std::min(pipe, w1);
+    const int first = g0 < w1 ? g0 : w;
+    char* rest = b.z + (g0 < w1 ? (size_t)g0 * per : 0);
+    const OrbScratch os(rest, (size_t)(b.z + (size_t)w1 * per - rest), p.n, o.ks);
+    launch_lisa(p.n, o.ks, ds->t0, ds->dt, b.lisa, os.cs, s);
     nl += 3;
     cudaStream_t so = ctx->pstream[0], sf = ctx->pstream[1];
     cudaEvent_t* ev = ctx->pev.data();
     cudaEventRecord(ev[0], s);
     cudaStreamWaitEvent(so, ev[0], 0);
     cudaStreamWaitEvent(sf, ev[0], 0);
-    // orbits: the first group's alone, then every other walker's in one
-    // launch that runs beside the first group's waveform (an orbit launch
-    // takes about as long for a few walkers as for a thousand: each walker's
-    // integration is sequential in time, so one launch per group would queue
-    // G of those latencies)
-    const int w1 = std::min(wave, w);
-    const int g0 = (w1 + std::min(pipe, w1) - 1) / std::min(pipe, w1);
-    orbit_of(0, g0, so);
+    if (first < w)
+      orbit_of(0, first, os.cs, b.z, (int64_t)((size_t)g0 * per / orbit_bytes(p.n, o.ks)), so);
+    else
+      orbit_of(0, w, os.cs, os.orb, os.fit, so);
     cudaEventRecord(ev[1], so);
-    if (g0 < w) orbit_of(g0, w - g0, so);
+    if (first < w) orbit_of(first, w - first, os.cs, os.orb, os.fit, so);
     cudaEventRecord(ev[3], so);
     int prev_gs = 0, prev_g = 0;   // group size and count of the previous wave
     for (int i0 = 0, wv = 0; i0 < w; i0 += wave, ++wv) {
@@ -836,24 +844,24 @@ extern "C" int emri_ak_waveform(emri_ctx* ctx, const emri_grid* grid, const doub
   Carve probe(nullptr);
   probe.take<WalkerC>(w);
   probe.take<Knot>((size_t)w * (nk + 1));
-  probe.take<char>((size_t)w * orbit_bytes(grid->n, o.ks));
   probe.take<char>(o.precision ? (size_t)w * nk * kIvMBytes : 0);
-  probe.take<double>(lisa_len(grid->n, o.ks));
+  probe.take<double>(lisa_len(grid->n));
   if ((rc = ctx->ws.reserve(ctx, probe.off + 512, s))) return rc;
   ctx->ws.acquire(s);
   Carve cv(ctx->ws.ptr);
   WalkerC* wc = cv.take<WalkerC>(w);
   Knot* kn = cv.take<Knot>((size_t)w * (nk + 1));
-  char* orb = cv.take<char>((size_t)w * orbit_bytes(grid->n, o.ks));
   char* ivs = cv.take<char>(o.precision ? (size_t)w * nk * kIvMBytes : 0);
-  double* lisa = cv.take<double>(lisa_len(grid->n, o.ks));
+  double* lisa = cv.take<double>(lisa_len(grid->n));
+  // the orbit step's own memory is the caller's output, written afterwards
+  const OrbScratch os(z_out, (size_t)w * grid->n * (o.precision ? sizeof(float2) : sizeof(double2)), grid->n, o.ks);
   Profiler* pf = &ctx->prof;
   { KTimer t(pf, EMRI_K_PROLOGUE, s); launch_prologue(theta, w, w, grid->n, grid->dt, o, ctx->gl, wc, s); }
-  launch_lisa(grid->n, o.ks, grid->t0, grid->dt, lisa, s);
+  launch_lisa(grid->n, o.ks, grid->t0, grid->dt, lisa, os.cs, s);
   int64_t nl = 0;
   {
     KTimer t(pf, EMRI_K_ORBIT, s);
-    nl = launch_orbit(wc, w, grid->n, grid->dt, lisa_knots(lisa, grid->n), o, kn, ctx->mcpi, orb, s);
+    nl = launch_orbit(wc, w, grid->n, grid->dt, os.cs, o, kn, ctx->mcpi, os.orb, os.fit, s);
   }
   if (o.precision) launch_intervals_mixed(kn, w, grid->n, o.ks, grid->dt, ivs, s);
   { KTimer t(pf, EMRI_K_WAVE, s); launch_wave(kn, wc, w, grid->n, grid->dt, grid->t0, o, z_out, true, ctx->bt, lisa, ivs, s); }

@@ -54,13 +54,12 @@ struct Carve {
 struct LoglikeBufs {
   WalkerC* wc;
   Knot* knots;
-  char* orb;       // orbit solver state [w][orbit_bytes]
   char* ivs;       // mixed interval records [w][n/ks]
-  double* lisa;    // LISA-phase table (lisa_len)
+  double* lisa;    // per-tile LISA-phase table [n/256][8]
   char* dtab;
   char* rtab;      // per-walker row delay factors [w][n2]
   double2* partial;
-  char* z;
+  char* z;         // time series [wave][n]; before them the orbit step's own memory (OrbScratch)
 };
 
 // Per-kernel event timing (enabled by emri_ctx_profile).

@@ -75,12 +75,30 @@ void launch_fdprop(const double* theta, int64_t ld, int w, int64_t n, double dt,
                    double fstar, const double* coef, int64_t ldc, FdW* fd, cudaStream_t s);
 
 // orbit: knots[w][nk+1], nk = n / ks
-// mcpi_tab: Chebyshev-Picard tables (qn then qk), required; orb: solver state
-// of the walkers, orbit_bytes(n, ks) each; cs: cos, sin of the LISA orbital
-// phase at the knots (lisa_knots).  Returns the number of launches.
+// mcpi_tab: Chebyshev-Picard tables (qn then qk), required; cs: cos, sin of the
+// LISA orbital phase at the knots (launch_lisa); orb: solver state of `fit`
+// walkers, orbit_bytes(n, ks) each, 16-byte aligned, free again afterwards
+// (more walkers than that take turns).  Returns the number of launches.
 int launch_orbit(WalkerC* wc, int w, int64_t n, double dt, const double2* cs, const OptsN& o, Knot* knots,
-                 const double* mcpi_tab, char* orb, cudaStream_t s);
+                 const double* mcpi_tab, char* orb, int64_t fit, cudaStream_t s);
 size_t orbit_bytes(int64_t n, int ks);
+
+// Memory that only the orbit step uses: the LISA phase table at the knots,
+// then the solver state.  It lies where the step's successors write the time
+// series; one series of n samples holds the table and one walker's state.
+struct OrbScratch {
+  double2* cs;
+  char* orb;
+  int64_t fit;   // walkers whose state fits
+  // in the `bytes` at p (alignment as the series': 8 bytes)
+  OrbScratch(void* p, size_t bytes, int64_t n, int ks) {
+    char* a = (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255);
+    const size_t tab = ((size_t)(n / ks + 1) * 16 + 255) & ~(size_t)255;
+    cs = (double2*)a;
+    orb = a + tab;
+    fit = (int64_t)((bytes - (size_t)(orb - (char*)p)) / orbit_bytes(n, ks));
+  }
+};
 
 // waveform: z[w][n] (double2 or float2); unit_scale multiplies by mu_s c (cm units)
 // lisa: LISA orbital phase table (launch_lisa); ivs: mixed
@@ -90,10 +108,9 @@ void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double 
                  cudaStream_t s);
 void launch_intervals_mixed(const Knot* knots, int w, int64_t n, int ks, double dt, void* ivs, cudaStream_t s);
 // cos, sin of the LISA orbital phase at the pattern-fit nodes of each
-// 256-sample tile, [n/256][8], then at the knots, [n/ks + 1][2]
-inline size_t lisa_len(int64_t n, int ks) { return (size_t)(n / 256) * 8 + (size_t)(n / ks + 1) * 2; }
-inline const double2* lisa_knots(const double* tab, int64_t n) { return (const double2*)(tab + (n / 256) * 8); }
-void launch_lisa(int64_t n, int ks, double t0, double dt, double* tab, cudaStream_t s);
+// 256-sample tile, tiles[n/256][8], and at the knots, knots[n/ks + 1]
+inline size_t lisa_len(int64_t n) { return (size_t)(n / 256) * 8; }
+void launch_lisa(int64_t n, int ks, double t0, double dt, double* tiles, double2* knots, cudaStream_t s);
 constexpr size_t kIvMBytes = 104;
 
 // FFT pass 1 (columns, with the inter-pass twiddle; out may be z); sign -1 forward, +1 inverse

@@ -1006,32 +1006,32 @@ __global__ void __launch_bounds__(32) k1f_tail(WalkerC* __restrict__ wcs, int64_
 size_t orbit_bytes(int64_t n, int ks) { return orb_walker_bytes(n / mcpi_segment(n, ks)); }
 
 int launch_orbit(WalkerC* wc, int w, int64_t n, double dt, const double2* cs, const OptsN& o, Knot* knots,
-                 const double* mcpi_tab, char* orb, cudaStream_t s) {
+                 const double* mcpi_tab, char* orb, int64_t fit, cudaStream_t s) {
   if (w <= 0) return 0;
   const int64_t seg = mcpi_segment(n, o.ks), ns = n / seg, nk = n / o.ks;
   const int K = (int)(seg / o.ks), back = o.mode == 1, pn = o.pn_terms;
   const double* qn = mcpi_tab;
   const double* qk = mcpi_tab + 32 * 32;
-  const size_t ob = orb_walker_bytes(ns);
   const int nsg = K >= 32 ? 1 : (int)((nk < 32 ? nk : 32) / K);
   int launches = 0;
-  // walkers on grid y of the segment kernels, at most kMaxGridY per launch
-  for (int w0 = 0; w0 < w; w0 += kMaxGridY) {
-    const int ww = w - w0 < kMaxGridY ? w - w0 : kMaxGridY;
+  // walkers on grid y of the segment kernels: at most kMaxGridY per launch, and
+  // no more than the solver state holds
+  const int step = (int)(fit < 1 ? 1 : fit < kMaxGridY ? fit : kMaxGridY);
+  for (int w0 = 0; w0 < w; w0 += step) {
+    const int ww = w - w0 < step ? w - w0 : step;
     WalkerC* c = wc + w0;
-    char* ow = orb + (size_t)w0 * ob;
     Knot* kn = knots + (int64_t)w0 * (nk + 1);
     const dim3 ge((unsigned)((ns + kEvalWarps - 1) / kEvalWarps), (unsigned)ww);
     const dim3 gk((unsigned)((nk + 31) / 32), (unsigned)ww);
-    k1a_coarse<<<ww, 32, 0, s>>>(c, n, dt, o.ks, pn, back, qn, ow);
-    k1b_eval<0><<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, ow);
-    k1b_eval<1><<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, ow);
-    k1b_eval<2><<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, ow);
-    k1b_eval<3><<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, ow);
-    k1c_final<<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, ow);
-    k1d_starts<<<ww, 32, (size_t)ns * 40, s>>>(n, o.ks, ow);
-    k1e_knots<<<gk, 32, (size_t)nsg * kRateStride * 8, s>>>(c, n, dt, cs, o.ks, pn, back, o.doppler, qk, ow, kn);
-    k1f_tail<<<ww, 32, 0, s>>>(c, n, dt, cs, o.ks, pn, back, o.doppler, qn, qk, ow, kn);
+    k1a_coarse<<<ww, 32, 0, s>>>(c, n, dt, o.ks, pn, back, qn, orb);
+    k1b_eval<0><<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, orb);
+    k1b_eval<1><<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, orb);
+    k1b_eval<2><<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, orb);
+    k1b_eval<3><<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, orb);
+    k1c_final<<<ge, 32 * kEvalWarps, 0, s>>>(c, n, dt, o.ks, pn, back, qn, orb);
+    k1d_starts<<<ww, 32, (size_t)ns * 40, s>>>(n, o.ks, orb);
+    k1e_knots<<<gk, 32, (size_t)nsg * kRateStride * 8, s>>>(c, n, dt, cs, o.ks, pn, back, o.doppler, qk, orb, kn);
+    k1f_tail<<<ww, 32, 0, s>>>(c, n, dt, cs, o.ks, pn, back, o.doppler, qn, qk, orb, kn);
     launches += 9;
   }
   return launches;

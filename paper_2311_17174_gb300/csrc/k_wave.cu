@@ -264,19 +264,19 @@ __global__ void k1b_intervals(const Knot* __restrict__ knots, int64_t nk, int ks
 
 // cos, sin of the LISA orbital phase phibar = 2 pi t / T: the four
 // pattern-fit nodes of each 256-sample tile (offsets 0, 256/3, 512/3, 256;
-// tab[8 tile + 2q] = cos, the next = sin), then the knots every ks samples.
+// tiles[4 tile + q]) and the knots every ks samples.
 // They are the same for every walker, and a sine and cosine cost ~50 FP64
 // instructions.
-__global__ void k_lisa(int64_t ntiles, int64_t nknots, int ks, double t0, double dt, double* __restrict__ tab) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 4 * ntiles + nknots) return;
-  const bool knot = i >= 4 * ntiles;
-  const double at = knot ? (double)((i - 4 * ntiles) * ks) : (double)((i >> 2) * 256) + 256.0 * (double)(i & 3) / 3.0;
+__global__ void k_lisa(int64_t ntiles, int64_t nknots, int ks, double t0, double dt, double2* __restrict__ tiles,
+                       double2* __restrict__ knots) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, k = i - 4 * ntiles;
+  if (k >= nknots) return;
+  const double at = k >= 0 ? (double)(k * ks) : (double)((i >> 2) * 256) + 256.0 * (double)(i & 3) / 3.0;
   double f = (t0 + at * dt) / kYear;
   f -= floor(f);
   double sn, cs;
   sincospi(2.0 * f, &sn, &cs);
-  reinterpret_cast<double2*>(tab)[i] = make_double2(cs, sn);
+  (k >= 0 ? knots[k] : tiles[i]) = make_double2(cs, sn);
 }
 
 void launch_intervals_mixed(const Knot* knots, int w, int64_t n, int ks, double dt, void* ivs, cudaStream_t s) {
@@ -290,9 +290,9 @@ void launch_intervals_mixed(const Knot* knots, int w, int64_t n, int ks, double 
   }
 }
 
-void launch_lisa(int64_t n, int ks, double t0, double dt, double* tab, cudaStream_t s) {
+void launch_lisa(int64_t n, int ks, double t0, double dt, double* tiles, double2* knots, cudaStream_t s) {
   const int64_t nt = n / 256, nkn = n / ks + 1;
-  k_lisa<<<(unsigned)((4 * nt + nkn + 127) / 128), 128, 0, s>>>(nt, nkn, ks, t0, dt, tab);
+  k_lisa<<<(unsigned)((4 * nt + nkn + 127) / 128), 128, 0, s>>>(nt, nkn, ks, t0, dt, (double2*)tiles, knots);
 }
 
 // --------------------------------------------------- response + harmonics
