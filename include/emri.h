@@ -255,10 +255,10 @@ int emri_fft_batch(emri_ctx* ctx, void* z_dev, int64_t n, int batch, int precisi
  * application hands it, a process whose device memory is fully reserved by
  * another allocator, or a real-time loop that must never enter the
  * allocator.  Same transform, layout and arguments as emri_fft_batch, but no
- * context: the scratch the second pass writes (32 MiB: at least one whole
+ * context: the scratch between the two passes (32 MiB: at least one whole
  * sequence, several when they are shorter) and the twiddle tables are
  * file-scope static device arrays of the library
- * (EMRI_NOALLOC_SCRATCH_BYTES of scratch plus 216 KiB of tables, held on
+ * (EMRI_NOALLOC_SCRATCH_BYTES of scratch plus 376 KiB of tables, held on
  * every GPU that loads the library until the process exits).  Nothing is
  * allocated by the call.
  *  - Limit: one sequence must fit the scratch, n * 16 B (FP64) or n * 8 B
@@ -266,9 +266,10 @@ int emri_fft_batch(emri_ctx* ctx, void* z_dev, int64_t n, int batch, int precisi
  *    n <= 2^22 in FP32; larger n returns EMRI_EINVAL with a message.  Any
  *    batch size is accepted (processed in chunks that fit the scratch).
  *  - The first call on a device (the current device) resolves the arrays'
- *    addresses with cudaGetSymbolAddress and fills the tables, synchronising
- *    `stream`; make that first call before any stream capture (a first call
- *    on a capturing stream returns EMRI_EINVAL and does nothing).
+ *    addresses with cudaGetSymbolAddress and fills the tables on `stream`,
+ *    synchronising it and no other; make that first call before any stream
+ *    capture (a first call on a capturing stream returns EMRI_EINVAL and does
+ *    nothing).
  *  - All calls on a device share the scratch: calls whose work overlaps on
  *    the GPU (different streams, unordered host threads) race. */
 #define EMRI_NOALLOC_SCRATCH_BYTES (32u << 20)

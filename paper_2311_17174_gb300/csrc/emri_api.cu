@@ -586,7 +586,7 @@ extern "C" int emri_ctx_create(int device, size_t budget, emri_ctx** out) {
   }
   launch_twiddle_init(c->tw, c->stream);
   cudaMemcpyAsync(c->gl, glh, sizeof glh, cudaMemcpyHostToDevice, c->stream);
-  const bool fft_ok = fft_setup();
+  const bool fft_ok = fft_setup(c->stream);
   e2 = cudaStreamSynchronize(c->stream);
   if (e2 == cudaSuccess && !fft_ok) e2 = cudaErrorUnknown;
   if (e2 == cudaSuccess) e2 = cudaGetLastError();

@@ -127,8 +127,9 @@ void launch_fft_pass2_ip(const void* y, int w, const FftPlan& p, bool fp32, cons
 // dh_scale / hh_scale undo the dataset's FP32 scaling (1 for FP64)
 void launch_finalize(const double2* partial, int n2, const WalkerC* wc, int w, double dh_scale, double hh_scale,
                      double* lnl, double* dh, double* hh, uint32_t* status, cudaStream_t s);
-// shared-memory limits and fixed-point tables on the current device; false on failure
-bool fft_setup();
+// shared-memory limits and fixed-point tables on the current device (the tables
+// on stream s); false on failure
+bool fft_setup(cudaStream_t s);
 
 // dataset preparation: the weighted conjugate spectrum g = w conj(D) and
 // the weights w in the pass-2 order (k2-major), plus FP32 copies scaled by

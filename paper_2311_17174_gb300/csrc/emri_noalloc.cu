@@ -15,8 +15,8 @@
 // fixed size, present on every GPU that loads the library until the process
 // exits.  Their device addresses are looked up once per device
 // (cudaGetSymbolAddress, with that device current) the first time the entry
-// point runs there; that first call also fills the twiddle tables and
-// synchronises the stream, so it must not be made while the stream is being
+// point runs there; that first call also fills the tables on the caller's
+// stream and synchronises it (no other), so it must not be made while the stream is being
 // captured (it is refused with EMRI_EINVAL then; later calls may be).
 // Nothing here calls cudaMalloc, cudaFree or an allocating
 // library routine.  Every call on a device shares the same scratch, so calls
@@ -80,7 +80,7 @@ int setup_device(int dev, cudaStream_t s, DevState** out) {
     st.tw.tc64 = (double2*)(t + 4096 * 16 + 1024 * 16 + 4096 * 8 + 1024 * 8);
     st.tw.tt32 = (float2*)(t + 4096 * 16 + 1024 * 16 + 4096 * 8 + 1024 * 8 + 4096 * 16);
     launch_twiddle_init(st.tw, s);
-    const bool fft_ok = fft_setup();
+    const bool fft_ok = fft_setup(s);
     e = cudaStreamSynchronize(s);
     if (e == cudaSuccess && !fft_ok) e = cudaErrorUnknown;
     if (e == cudaSuccess) e = cudaGetLastError();

@@ -43,9 +43,10 @@ FX_HD int4 pack(i64 c, i64 s) {
   return make_int4(a.h, a.l, b.h, b.l);
 }
 
-// Fills the tables of the current device from long double values (a second
-// context's upload rewrites them unchanged).
-static bool upload_tables() {
+// Fills the tables of the current device on stream s, which nothing else waits
+// for, from long double values kept by the process (a second context's upload
+// rewrites them unchanged).
+static bool upload_tables(cudaStream_t s) {
   static const std::vector<int4> host = [] {
     std::vector<int4> t;
     auto put = [&](long double turns) {
@@ -67,10 +68,11 @@ static bool upload_tables() {
     }
     return t;
   }();
-  return cudaMemcpyToSymbol(g_trig, trig.data(), sizeof(g_trig)) == cudaSuccess &&
-         cudaMemcpyToSymbol(g_stage, host.data(), sizeof(g_stage)) == cudaSuccess &&
-         cudaMemcpyToSymbol(g_ta, host.data() + kStageLen, sizeof(g_ta)) == cudaSuccess &&
-         cudaMemcpyToSymbol(g_tb, host.data() + kStageLen + 4096, sizeof(g_tb)) == cudaSuccess;
+  const auto put = [s](const auto& symbol, const void* src) {
+    return cudaMemcpyToSymbolAsync(symbol, src, sizeof(symbol), 0, cudaMemcpyHostToDevice, s) == cudaSuccess;
+  };
+  return put(g_trig, trig.data()) && put(g_stage, host.data()) && put(g_ta, host.data() + kStageLen) &&
+         put(g_tb, host.data() + kStageLen + 4096);
 }
 
 struct Z {

@@ -1383,13 +1383,13 @@ void launch_inner_dd(const double2* d, const double* w, int64_t n, double* out, 
 }
 
 // Raises the dynamic shared-memory limit of the FFT kernels and uploads the
-// fixed-point tables (once per device); false on failure.
+// fixed-point tables on stream s (once per device); false on failure.
 template <typename F>
 static void raise(F f) {
   cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
-bool fft_setup() {
+bool fft_setup(cudaStream_t s) {
   raise(k3_pass1_r8<8, 8>), raise(k3_pass1_r8<9, 8>);
   raise(k3_pass1<float2, 10, FftCfg<float2>::kCols>);
   raise(k4_pass2_store<float2, 5>), raise(k4_pass2_store<float2, 6>), raise(k4_pass2_store<float2, 7>);
@@ -1410,7 +1410,7 @@ bool fft_setup() {
 #define P3(L) raise(k4_pass2_ip_r8<L, false>), raise(k4_pass2_ip_r8<L, true>)
   P3(8); P3(9); P3(10); P3(11); P3(12);
 #undef P3
-  return fxfft::upload_tables();
+  return fxfft::upload_tables(s);
 }
 
 }  // namespace emri
