@@ -356,20 +356,20 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   // ~800 FP64 instructions in double-double) and only pass 2 needs them and
   // their tables: on the side stream they run beside the orbit, whose launches
   // leave most of the GPU idle in a small call (8 walkers x 2^16: 191 -> 170 us).
-  side = side && pipe <= 1 && ctx->side;
+  side = side && pipe <= 1 && ctx->side.stream;
   {
     KTimer t(pf, EMRI_K_PROLOGUE, s);
-    if (side) cudaEventRecord(ctx->side_ev[0], s);
+    if (side) cudaEventRecord(ctx->side.ev[0], s);
     launch_prologue(theta, ld, w, p.n, ds->dt, o, ctx->gl, b.wc, s, side ? ProPart::kNoDelay : ProPart::kAll);
   }
   {
-    cudaStream_t sd = side ? ctx->side : s;
-    if (side) cudaStreamWaitEvent(sd, ctx->side_ev[0], 0);
+    cudaStream_t sd = side ? ctx->side.stream : s;
+    if (side) cudaStreamWaitEvent(sd, ctx->side.ev[0], 0);
     KTimer t(pf, EMRI_K_DELAY, sd);
     if (side) launch_prologue(theta, ld, w, p.n, ds->dt, o, ctx->gl, b.wc, sd, ProPart::kDelay);
     launch_delay_table(b.wc, w, p.n1, p.n2, f32, b.dtab, b.rtab, sd);
     if (side) {
-      cudaEventRecord(ctx->side_ev[1], sd);
+      cudaEventRecord(ctx->side.ev[1], sd);
       ++nl;
     }
   }
@@ -381,7 +381,7 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
     for (int i0 = 0; i0 < w; i0 += wave) {
       const int ww = std::min(wave, w - i0);
       wave_of(i0, ww, b.z, s);
-      if (side && i0 == 0) cudaStreamWaitEvent(s, ctx->side_ev[1], 0);
+      if (side && i0 == 0) cudaStreamWaitEvent(s, ctx->side.ev[1], 0);
       passes(i0, ww, b.z, s);
       nl += 4;
     }
@@ -598,11 +598,7 @@ extern "C" int emri_ctx_create(int device, size_t budget, emri_ctx** out) {
     delete c;
     return cuda_err(e2, "context tables");
   }
-  // without them the delay tables stay on the caller's stream
-  if (cudaEventCreateWithFlags(&c->side_ev[0], cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->side_ev[1], cudaEventDisableTiming) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess)
-    c->side = nullptr;
+  c->side.create();   // optional
   c->launches = 2;
   *out = c;
   return EMRI_OK;
@@ -622,9 +618,7 @@ extern "C" int emri_ctx_destroy(emri_ctx* c) {
     if (st) cudaStreamDestroy(st);
   for (cudaEvent_t e : c->pev)
     if (e) cudaEventDestroy(e);
-  if (c->side) cudaStreamDestroy(c->side);
-  for (cudaEvent_t e : c->side_ev)
-    if (e) cudaEventDestroy(e);
+  c->side.destroy();
   cudaStreamDestroy(c->stream);
   delete c;
   return EMRI_OK;

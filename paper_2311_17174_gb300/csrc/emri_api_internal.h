@@ -11,6 +11,7 @@
 
 #include "../../include/emri.h"
 #include "emri_internal.h"
+#include "side_stream.h"
 
 namespace emri {
 struct Server;
@@ -133,10 +134,7 @@ struct emri_ctx {
   int pipe[2] = {1, 0};
   cudaStream_t pstream[2] = {nullptr, nullptr};
   std::vector<cudaEvent_t> pev;
-  // side stream of a likelihood call's delay constants and tables, and the
-  // events of its fork and join (used under mu)
-  cudaStream_t side = nullptr;
-  cudaEvent_t side_ev[2] = {nullptr, nullptr};
+  emri::SideStream side;   // used under mu
 };
 
 struct emri_dataset {

@@ -21,7 +21,8 @@ def load(name):
     if inc is None:
         pytest.skip("no CUDA headers")
     out = os.path.join(tempfile.mkdtemp(prefix="emri_host_"), name + ".so")
-    r = subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, "-I", inc,
-                        os.path.join(HERE, name + ".cpp"), "-o", out], capture_output=True, text=True)
+    # -Bsymbolic: a harness's own fakes, not the CUDA runtime that torch has loaded
+    r = subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", CSRC,
+                        "-I", inc, os.path.join(HERE, name + ".cpp"), "-o", out], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     return ctypes.CDLL(out)
