@@ -192,8 +192,9 @@ enum emri_kernel {
 };
 
 /* Enable (1) or disable (0) per-kernel timing on this context and reset the
- * accumulators.  While enabled, every launch of the likelihood path is
- * bracketed by CUDA events recorded on the stream it is launched on.  Under
+ * accumulators.  While enabled, the launches of each step (kind) of the
+ * likelihood path are bracketed by CUDA events recorded on the stream they are
+ * launched on; the delay tables' stream runs beside the orbit's.  Under
  * the pipelined schedule (emri_ctx_set_pipeline) kernels of different walker
  * groups run at the same time, so a launch's interval also covers the
  * kernels beside it; set groups to 1 for a per-kernel breakdown. */

@@ -338,11 +338,12 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   auto orbit_of = [&](int j0, int gw, const double2* lk, char* orb, int64_t fit, cudaStream_t st) {
     Knot* kj = b.knots + (size_t)j0 * (nk + 1);
     KTimer t(pf, EMRI_K_ORBIT, st);
-    nl += launch_orbit(b.wc + j0, gw, p.n, ds->dt, lk, o, kj, ctx->mcpi, orb, fit, st);
+    t.launches = launch_orbit(b.wc + j0, gw, p.n, ds->dt, lk, o, kj, ctx->mcpi, orb, fit, st);
     if (f32) {
       launch_intervals_mixed(kj, gw, p.n, o.ks, ds->dt, b.ivs + (size_t)j0 * nk * kIvMBytes, st);
-      ++nl;
+      ++t.launches;
     }
+    nl += t.launches;
   };
   if (pipe == 0) {
     // by size: two groups when each holds at least 2^30 samples (walkers x
@@ -370,6 +371,7 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
     launch_delay_table(b.wc, w, p.n1, p.n2, f32, b.dtab, b.rtab, sd);
     if (side) {
       cudaEventRecord(ctx->side.ev[1], sd);
+      ++t.launches;
       ++nl;
     }
   }
@@ -471,11 +473,11 @@ cudaEvent_t Profiler::begin(cudaStream_t s) {
   return e;
 }
 
-void Profiler::end(int kind, cudaEvent_t b, cudaStream_t s) {
+void Profiler::end(int kind, cudaEvent_t b, cudaStream_t s, int launches) {
   std::lock_guard<std::mutex> lk(mu);
   cudaEvent_t e = get();
   cudaEventRecord(e, s);
-  pending.emplace_back(kind, b, e);
+  pending.emplace_back(kind, b, e, launches);
 }
 
 void Profiler::drain() {
@@ -485,7 +487,7 @@ void Profiler::drain() {
     float m = 0.f;
     cudaEventElapsedTime(&m, std::get<1>(t), std::get<2>(t));
     ms[std::get<0>(t)] += m;
-    count[std::get<0>(t)] += 1;
+    count[std::get<0>(t)] += std::get<3>(t);
     pool.push_back(std::get<1>(t));
     pool.push_back(std::get<2>(t));
   }
@@ -855,7 +857,7 @@ extern "C" int emri_ak_waveform(emri_ctx* ctx, const emri_grid* grid, const doub
   int64_t nl = 0;
   {
     KTimer t(pf, EMRI_K_ORBIT, s);
-    nl = launch_orbit(wc, w, grid->n, grid->dt, os.cs, o, kn, ctx->mcpi, os.orb, os.fit, s);
+    nl = t.launches = launch_orbit(wc, w, grid->n, grid->dt, os.cs, o, kn, ctx->mcpi, os.orb, os.fit, s);
   }
   if (o.precision) launch_intervals_mixed(kn, w, grid->n, o.ks, grid->dt, ivs, s);
   { KTimer t(pf, EMRI_K_WAVE, s); launch_wave(kn, wc, w, grid->n, grid->dt, grid->t0, o, z_out, true, ctx->bt, lisa, ivs, s); }

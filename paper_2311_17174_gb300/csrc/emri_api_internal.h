@@ -67,29 +67,30 @@ struct LoglikeBufs {
 struct Profiler {
   std::atomic<bool> on{false};
   std::mutex mu;
-  std::vector<std::tuple<int, cudaEvent_t, cudaEvent_t>> pending;
+  std::vector<std::tuple<int, cudaEvent_t, cudaEvent_t, int>> pending;   // kind, begin, end, launches
   std::vector<cudaEvent_t> pool;
   double ms[EMRI_NKERNEL] = {};
   int64_t count[EMRI_NKERNEL] = {};
   cudaEvent_t get();
-  // bracket one launch: begin() before, end() after
+  // bracket one step's launches: begin() before, end() after
   cudaEvent_t begin(cudaStream_t s);
-  void end(int kind, cudaEvent_t b, cudaStream_t s);
+  void end(int kind, cudaEvent_t b, cudaStream_t s, int launches);
   void drain();
   void reset();
 };
 
-// RAII helper: times one launch when profiling is on
+// RAII helper: times one step's launches when profiling is on
 struct KTimer {
   Profiler* p;
   int kind;
   cudaStream_t s;
+  int launches = 1;
   cudaEvent_t b = nullptr;
   KTimer(Profiler* p_, int k, cudaStream_t s_) : p(p_), kind(k), s(s_) {
     if (p && p->on) b = p->begin(s);
   }
   ~KTimer() {
-    if (b) p->end(kind, b, s);
+    if (b) p->end(kind, b, s, launches);
   }
 };
 
