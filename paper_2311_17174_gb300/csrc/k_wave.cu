@@ -1121,10 +1121,15 @@ void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double 
   (o.ks >= kBlk ? k2_wave_mixed<SEG, TH, true> : k2_wave_mixed<SEG, TH, false>)<<<grid, TH, 0, s>>>(                   \
       kn, wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
       // four warps a CTA where all CTA slots (six an SM) are taken, eight
-      // where they are not; a sample's result is the same
-      if (seg == 4096 && n / seg * ww >= 6 * 152) EMRI_WAVE_MIXED(4096, 128);
+      // where they are not; a sample's result is the same.  The shorter the
+      // segment, the more its set-up waits for: 1024 walkers x 2^15 (2048
+      // samples) 0.358 -> 0.301 ms, 2048 x 2^14 (1024) 0.452 -> 0.346 ms.
+      const bool full = n / seg * ww >= 6 * 152;
+      if (seg == 4096 && full) EMRI_WAVE_MIXED(4096, 128);
       else if (seg == 4096) EMRI_WAVE_MIXED(4096, 256);
+      else if (seg == 2048 && full) EMRI_WAVE_MIXED(2048, 128);
       else if (seg == 2048) EMRI_WAVE_MIXED(2048, 256);
+      else if (full) EMRI_WAVE_MIXED(1024, 128);
       else EMRI_WAVE_MIXED(1024, 256);
 #undef EMRI_WAVE_MIXED
     }
