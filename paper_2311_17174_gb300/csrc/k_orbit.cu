@@ -222,16 +222,21 @@ __device__ bool rk4_span(const OrbSrc& s, const WalkerC& c, OrbState& y, int64_t
 // int_0^{q/128} l_j, q = 0..128 (knot positions of the finest knot grid).
 // Built on the host.
 constexpr int kSeg = 65536;        // most samples per segment
-constexpr int kSegLeast = 4096;    // segments are not cut below this for parallelism alone
+// for parallelism alone, segments are not cut below so many samples and knots
+constexpr int kSegLeast = 4096, kSegKnots = 32;
 
 // Samples per segment (a power of two): at most 65536 and 128 knot intervals
 // (the knot-weight table has 129 rows), and short enough for eight segments
-// per walker as long as they keep 4096 samples, so that a small call's
-// segments spread over the GPU.
+// per walker as long as they keep 4096 samples and 32 knots, so that a small
+// call's segments spread over the GPU.  A segment costs the same work whatever
+// its length (32 nodes), which counts once walkers fill the GPU: at K_s = 1024,
+// 1024 walkers x 2^15 take 0.20 ms in one segment each and 0.51 in eight, 8
+// walkers x 2^16 0.099 in two and 0.107 in eight.
 __host__ __device__ __forceinline__ int64_t mcpi_segment(int64_t n, int ks) {
   int64_t seg = kSeg;
   if (seg > 128 * (int64_t)ks) seg = 128 * (int64_t)ks;
-  while (seg > kSegLeast && 8 * seg > n) seg >>= 1;
+  const int64_t least = kSegLeast > (int64_t)kSegKnots * ks ? kSegLeast : (int64_t)kSegKnots * ks;
+  while (seg > least && 8 * seg > n) seg >>= 1;
   if (seg > n) seg = n;
   return seg;
 }
