@@ -227,13 +227,29 @@ __host__ __device__ inline dd dd_asinh(dd a) {
   return dd_log(dd_add(a, s));
 }
 
-// fractional part in [0, 1) of a dd value
+// fractional part in [0, 1) of a dd value, to dd precision (just below an
+// integer it is (1, -x): the sum is below one).  hi - floor(hi) is not a double
+// where -1/2 < hi < 0, so it is taken as a sum.
 __host__ __device__ inline dd dd_frac(dd a) {
-  double f = floor(a.hi);
-  dd r = dd_add_d(dd{a.hi - f, 0.0}, a.lo);   // a.hi - f is exact
+  dd r = dd_add_d(two_sum(a.hi, -floor(a.hi)), a.lo);
   if (r.hi < 0.0) r = dd_add_d(r, 1.0);
-  if (r.hi >= 1.0) r = dd_add_d(r, -1.0);
+  if (r.hi > 1.0 || (r.hi == 1.0 && r.lo >= 0.0)) r = dd_add_d(r, -1.0);
   return r;
+}
+
+// dd fraction x in [0, 1) -> 128-bit fixed point (hi, lo) = x 2^128, mod 2^128.
+// x.hi 2^64 is exact but carries only 53 bits; the low bits of the 64-bit
+// integer part come from x.lo 2^64, which can reach ~2^11 in magnitude, so
+// its integer part is carried into hi and only its fraction goes to lo.
+__host__ __device__ inline void dd_to_fx128(dd x, unsigned long long& hi, unsigned long long& lo) {
+  const double two64 = 18446744073709551616.0;
+  const double t = x.hi * two64;            // exact scaling, 0 <= t <= 2^64
+  const double H = floor(t);                // exact
+  const double r = (t - H) + x.lo * two64;  // t - H and x.lo 2^64 exact; |r| < ~2^12
+  const double F = floor(r);                // exact integer
+  const double rem = r - F;                 // [0, 1]
+  hi = (t < two64 ? (unsigned long long)H : 0ull) + (unsigned long long)(long long)F;   // mod 2^64
+  lo = rem < 1.0 ? (unsigned long long)(rem * two64) : ~0ull;
 }
 
 // Compensated accumulation of x into the unevaluated sum hi + lo.

@@ -236,8 +236,6 @@ __global__ void __launch_bounds__(128) k0_prologue(const double* __restrict__ th
 // m r mod 1 from two 64-bit integer products (exact), its top 32 bits as the
 // phase in [-1/2, 1/2) cycles, then the FP32 sincospif; no FP64 operation
 // per entry.  The FP64 tables take it in double-double and FP64 sincospi.
-__device__ void dd_to_fx128(dd x, unsigned long long& hi, unsigned long long& lo);
-
 template <typename C2>
 __global__ void k0_delay_table(const WalkerC* __restrict__ wc, int n1, int n2, C2* __restrict__ tab,
                                C2* __restrict__ rtab) {
@@ -330,21 +328,6 @@ void launch_prologue_export(const WalkerC* wc, int w, double* out, cudaStream_t 
 }
 
 // ----------------------------------------- frequency-dependent propagation
-// dd fraction x in [0, 1) -> 128-bit fixed point (hi, lo) = x 2^128, mod 2^128.
-// x.hi 2^64 is exact but carries only 53 bits; the low bits of the 64-bit
-// integer part come from x.lo 2^64, which can reach ~2^11 in magnitude, so
-// its integer part is carried into hi and only its fraction goes to lo.
-__device__ void dd_to_fx128(dd x, unsigned long long& hi, unsigned long long& lo) {
-  const double two64 = 18446744073709551616.0;
-  const double t = x.hi * two64;            // exact scaling, 0 <= t < 2^64
-  const double H = floor(t);                // exact
-  const double r = (t - H) + x.lo * two64;  // t - H and x.lo 2^64 exact; |r| < ~2^12
-  const double F = floor(r);                // exact integer
-  const double rem = r - F;                 // exact, [0, 1)
-  hi = (unsigned long long)H + (unsigned long long)(long long)F;   // mod 2^64
-  lo = (unsigned long long)(rem * two64);
-}
-
 // beta_m = -(t_LB/2) b_m df^(m+1) / f_*^m (cycles per |k|^(m+1)), reduced mod 1
 // in dd before the conversion to fixed point.
 __global__ void k0_fdprop(const double* __restrict__ theta, int64_t ld, int w, int64_t n, double dt, ProConst K, int qm, int qt, double fstar, const double* __restrict__ coef, int64_t ldc,
