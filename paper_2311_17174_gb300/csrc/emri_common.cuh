@@ -191,7 +191,7 @@ __host__ __device__ __forceinline__ dd dd_sqrt(dd a) {
 }
 
 // exp of a dd argument: x = k ln2 + r, r reduced by 2^-9 (|r| < 6.8e-4),
-// exp(r) - 1 by its Taylor series -- in dd up to r^4, the rest, below 1e-15 of
+// exp(r) - 1 by its Taylor series -- in dd up to r^4, the rest, below 1.9e-15 of
 // the sum, in double -- then 9 squarings and the 2^k scale.  Relative error
 // ~1e-31.
 __host__ __device__ inline dd dd_exp(dd x) {

@@ -20,12 +20,9 @@ typedef unsigned long long u64;
 
 #define FX_HD __host__ __device__ __forceinline__
 
-// a b + c, one multiply-add (32 x 32 + 64 -> 64 bits).  The product is written
-// as an instruction: an operand known to be non-negative is otherwise widened
-// without its sign, and its product with a signed one takes three.  The sum is
-// not (mad.wide), which the assembler splits into product and sum about half
-// of the time.  128 walkers x 2^21, n_max 20, waveform kernel: 50.0 ms from
-// the C expression, 32.8 ms as mad.wide, 30.8 ms like this.
+// a b + c (32 x 32 + 64 -> 64 bits).  Waveform kernel, 128 walkers x 2^21, n_max
+// 20: 50.0 ms with the C expression, 32.8 ms with mad.wide, 30.8 ms with
+// mul.wide and a C sum.
 FX_HD i64 wide(int a, int b, i64 c) {
 #ifdef __CUDA_ARCH__
   i64 r;

@@ -729,8 +729,9 @@ struct WaveSmem {
 // instructions, 20000 cycles, that few threads have work for in a single
 // segment; four segments fill the CTA's warps with it and pay its latency once
 // (56.7 -> 49.2 ms when the sums were slower).  A segment's result does not
-// depend on kSub.  Three CTAs per SM at 80 registers: 30.8 -> 30.1 ms against
-// two at 126, 16 sources x 2^16 0.141 -> 0.128 ms.
+// depend on kSub.  Three CTAs per SM at 80 registers, with spills of 64 (kSub =
+// 1) and 52 bytes, against two at 126: 30.8 -> 30.1 ms, 16 sources x 2^16 0.141
+// -> 0.128 ms.
 template <int kSub>
 __global__ void __launch_bounds__(kTile, 3) k2_wave_f64(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
                                                         int64_t n, double dt, double t0, int ks, int n_max,
@@ -827,13 +828,8 @@ __global__ void __launch_bounds__(kTile, 3) k2_wave_f64(const Knot* __restrict__
   __syncthreads();
   for (int i = t; i < 9 * kSub * n_max; i += kTile) {
     const int sub = i / (9 * n_max), r = i % (9 * n_max), m = r / 9, f = (r % 9) / 3, p = r % 3;
-    const int span = tile_span(j0 + sub * kSegF, jplunge, kSegF);
-    double v = S.bq[sub][r];
-    if (span != kSegF) {       // the fit's time to rho = r / 1024
-      const double rs = (double)kSegF / (double)span;
-      v *= p == 0 ? 1.0 : p == 1 ? rs : rs * rs;
-    }
-    harm_put(S.hx[sub][m], m, f, p, v, S.hsc[sub]);
+    const HarmScale hs = S.hsc[sub];
+    harm_put(S.hx[sub][m], m, f, p, S.bq[sub][r], hs, tile_span(j0 + sub * kSegF, jplunge, kSegF));
   }
   if (t >= 256 - 4 * kTiles && !exact_f) {   // pattern q of tile tt, in the sums' unit
     const int i = t - (256 - 4 * kTiles), tt = i / 4, q = i % 4;
@@ -897,7 +893,8 @@ __global__ void __launch_bounds__(kTile, 3) k2_wave_f64(const Knot* __restrict__
 // a sample at n_max = 20 (114 paired with the quadratics evaluated per sample,
 // 35.0 -> 33.8 ms for 1024 walkers x 2^21).  kOneIv (K_s >= 128): the block's
 // four samples share one interval record; with it and 24 warps per SM at 80
-// registers 33.2 -> 32.8 ms (at 64 registers it spills: 34.1 ms).
+// registers 33.2 -> 32.8 ms, although it then spills 72 bytes (stores; 92 of
+// loads) that two records do not; at 64 registers it spills more: 34.1 ms.
 // The set-up's barriers leave the other warps of a CTA idle: with four warps a
 // CTA instead of eight 33.8 -> 33.3 ms (333 walkers x 2^18: 0.894 -> 0.869 ms);
 // a call that does not fill the GPU keeps eight (8 walkers x 2^16: 16 against
@@ -907,7 +904,7 @@ __global__ void __launch_bounds__(kTile, 3) k2_wave_f64(const Knot* __restrict__
 // LISA orbital phase step per sample [cycles] for them.  No FP64 instruction
 // runs per thread: e0 is tested once per CTA.
 template <int kSegM, int kMixThreads, bool kOneIv>
-__global__ void __launch_bounds__(kMixThreads, 768 / kMixThreads) k2_wave_mixed(const Knot* __restrict__ knots, const WalkerC* __restrict__ wcs,
+__global__ void __launch_bounds__(kMixThreads, 768 / kMixThreads) k2_wave_mixed(const WalkerC* __restrict__ wcs,
                                                           int64_t n, int exact_f, float dphib, int ks, int n_max,
                                                           float2* __restrict__ z, int unit_scale,
                                                           const float* __restrict__ bc, const float* __restrict__ ifact,
@@ -1119,7 +1116,7 @@ void launch_wave(const Knot* knots, const WalkerC* wc, int w, int64_t n, double 
       const int us = unit_scale ? 1 : 0;
 #define EMRI_WAVE_MIXED(SEG, TH)                                                                                       \
   (o.ks >= kBlk ? k2_wave_mixed<SEG, TH, true> : k2_wave_mixed<SEG, TH, false>)<<<grid, TH, 0, s>>>(                   \
-      kn, wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
+      wc + w0, n, ef, dpb, o.ks, o.n_max, zz, us, bt.c32, bt.f32, lisa, iv)
       // four warps a CTA where all CTA slots (six an SM) are taken, eight
       // where they are not; a sample's result is the same.  The shorter the
       // segment, the more its set-up waits for: 1024 walkers x 2^15 (2048

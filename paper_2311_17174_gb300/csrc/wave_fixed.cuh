@@ -58,10 +58,15 @@ FX_HD double pow2d(int k) {
 #endif
 }
 
-// Coefficient p (of rho^p) of quantity f (a, b, c) of harmonic index m, value v
-FX_HD void harm_put(HarmX& o, int m, int f, int p, double v, const HarmScale& hs) {
+// Coefficient p of quantity f (a, b, c) of harmonic index m: v, of (r/span)^p
+FX_HD void harm_put(HarmX& o, int m, int f, int p, double v, const HarmScale& hs, int span) {
   if ((m + 1) & 2) v = -v;   // the signs of the recurrence
-  const fx::i64 q = llrint(v * pow2d(p == 0 ? hs.k0 : p == 1 ? hs.k1 : hs.k2));
+  v *= pow2d(p == 0 ? hs.k0 : p == 1 ? hs.k1 : hs.k2);
+  if (span != 1024) {        // to rho = r / 1024
+    const double rs = 1024.0 / (double)span;
+    v *= p == 0 ? 1.0 : p == 1 ? rs : rs * rs;
+  }
+  const fx::i64 q = llrint(v);
   int* oh = p < 2 ? reinterpret_cast<int*>(&o) + 4 * f + 2 * p : o.h2 + f;
   int* ol = p < 2 ? oh + 1 : o.l2 + f;
   const bool one = p == 2 && !hs.two;

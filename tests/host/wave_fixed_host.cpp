@@ -67,7 +67,7 @@ extern "C" int harmonic_errors(const double* q, int n_max, const uint64_t* p, co
   std::vector<HarmX> hx(n_max);
   for (int m = 0; m < n_max; ++m)
     for (int f = 0; f < 3; ++f)
-      for (int k = 0; k < 3; ++k) harm_put(hx[m], m, f, k, q[9 * m + 3 * f + k], hs);
+      for (int k = 0; k < 3; ++k) harm_put(hx[m], m, f, k, q[9 * m + 3 * f + k], hs, 1024);
   for (int i = 0; i < count; ++i) {
     const fx::Trig cs = fx::sincos_cycles(p[i], table());
     fx::i64 C, S, R;
