@@ -233,6 +233,10 @@ size_t loglike_layout(const FftPlan& p, const OptsN& o, int w, int wave, Carve* 
   Carve dummy(nullptr);
   Carve& cv = c ? *c : dummy;
   LoglikeBufs t;
+  // the series first, at the allocation's start: at an odd multiple of 256 bytes
+  // pass 1's strided rows are slower (1024 mixed walkers x 2^21 7.84 against
+  // 7.68 ms, 128 in FP64 3.894 against 3.888)
+  t.z = cv.take<char>((size_t)wave * p.n * cs);
   t.wc = cv.take<WalkerC>(w);
   t.knots = cv.take<Knot>((size_t)w * (nk + 1));
   t.ivs = cv.take<char>(o.precision ? (size_t)w * nk * kIvMBytes : 0);
@@ -240,7 +244,6 @@ size_t loglike_layout(const FftPlan& p, const OptsN& o, int w, int wave, Carve* 
   t.dtab = cv.take<char>((size_t)w * p.n1 * cs);
   t.rtab = cv.take<char>((size_t)w * p.n2 * cs);
   t.partial = cv.take<double2>((size_t)w * p.n2);
-  t.z = cv.take<char>((size_t)wave * p.n * cs);
   if (b) *b = t;
   return cv.off + 256;
 }
@@ -347,9 +350,9 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   };
   if (pipe == 0) {
     // by size: two groups when each holds at least 2^30 samples (walkers x
-    // n).  On the 1024-walker 2^21 mixed step two groups take 44.5 against
-    // 45.3 ms; smaller groups lose more to the extra orbit launch and the
-    // stream hand-offs than the overlap gains (8 walkers: 2.5 -> 4.4 ms).
+    // n).  On the 1024-walker 2^21 mixed step two groups take 41.72 against
+    // 41.74 ms; smaller groups lose more to the extra orbit launch and the
+    // stream hand-offs than the overlap gains (8 walkers: 0.49 -> 0.56 ms).
     const int64_t w1 = std::min(wave, w);
     pipe = w1 * p.n >= ((int64_t)1 << 31) ? 2 : 1;
   }
