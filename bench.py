@@ -42,6 +42,10 @@ MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # 152 SMs x 2 FP64 FMA/clk (resp. 128 FP32 FMA/clk) x 2 flop x 2.07 GHz.
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
+# 32 x 32 + 64-bit integer multiply-adds: one per 4 cycles for a warp on an SM
+# sub-partition (probe, profiles/ncu_fixed_point_32w_2p20.md), 32 lanes, 4 x 152
+# sub-partitions at 2.07 GHz.
+INT_MAD_PEAK_T = 152 * 4 * 32 / 4 * 2.07e9 / 1e12
 
 
 # walker groups whose orbits, waveforms and FFT passes overlap in the mixed
@@ -336,11 +340,13 @@ def serve_bench(ctx, dsets, precision: int, rate: float, duration: float, n_max:
 
 
 # DRAM bytes per sample of k2_wave_f64 from one ncu capture of the kernel
-# (64 walkers x 2^20 samples, n_max 20: 69.54 MB read + 1013.18 MB written;
-# profiles/ncu_k2_wave_f64_64w_2p20.md, the kernel with 1024-sample segments),
-# scaled to a launch by the samples it processes (the kernel's traffic is its
-# 16-byte output per sample plus the per-segment orbit records, both
-# proportional to walkers x samples).
+# (64 walkers x 2^20 samples, n_max 20: 68.87 MB read + 1021.03 MB written;
+# profiles/ncu_fixed_point_32w_2p20.md), scaled to a launch by the samples it
+# processes (the kernel's traffic is its 16-byte output per sample plus the
+# per-segment orbit records, both proportional to walkers x samples).
+K2_FIXED_DRAM_BYTES_PER_SAMPLE = (68.874e6 + 1021.028e6) / (64 * 2 ** 20)
+# The same of its double-precision form (69.54 MB read + 1013.18 MB written;
+# profiles/ncu_k2_wave_f64_64w_2p20.md), for comparison.
 K2_F64_DRAM_BYTES_PER_SAMPLE = (69.544e6 + 1013.184e6) / (64 * 2 ** 20)
 
 
@@ -550,6 +556,15 @@ def flop_model(n_max: int) -> float:
     return 24.0 * n_max + 172.0
 
 
+def int_mad_model(n_max: int) -> float:
+    """32 x 32 + 64-bit multiply-adds per sample of the FP64 waveform kernel
+    (csrc/wave_fixed.cuh): 29 per harmonic (advancing cosine and sine 8, the
+    constant and linear coefficients 9 each, the quadratic ones 3) plus 221 per
+    sample (scaling the sums 12, three phases 27, three sines and cosines 87,
+    response 95)."""
+    return 29.0 * n_max + 221.0
+
+
 # ------------------------------------------------------------ CPU oracle
 def oracle_sample(theta, wl, data_fd, psd, walkers: int, threads: int):
     import oracle as O
@@ -752,15 +767,18 @@ def main():
         avg_ms = ktimes["wave"][0] / launches_wave
         walkers_per_launch = W * args.steps / launches_wave
         flops = flop_model(wl.n_max) * wl.n * walkers_per_launch
-        achieved = flops / (avg_ms / 1e3) / 1e12
-        traffic = K2_F64_DRAM_BYTES_PER_SAMPLE * wl.n * walkers_per_launch if wl.n_max == 20 else None
-        roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP64_PEAK_TFLOPS, "traffic": traffic, "kernel": "k2_wave_f64",
-                "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 x 2.07 GHz (FP64 vector unit); the kernel "
-                               "computes in 64-bit fixed point on the integer pipe, so the fraction passes 1",
-                "flops_per_launch": flops, "avg_launch_ms": avg_ms}
+        mads = int_mad_model(wl.n_max) * wl.n * walkers_per_launch
+        achieved = mads / (avg_ms / 1e3) / 1e12
+        traffic = K2_FIXED_DRAM_BYTES_PER_SAMPLE * wl.n * walkers_per_launch if wl.n_max == 20 else None
+        roof = {"bound": "alu", "achieved": achieved, "peak": INT_MAD_PEAK_T, "unit": "T multiply-add/s",
+                "frac": achieved / INT_MAD_PEAK_T, "traffic": traffic, "kernel": "k2_wave_f64",
+                "peak_source": "32 x 32 + 64-bit integer multiply-adds, one per 4 cycles and SM sub-partition for a "
+                               "warp (probe): 152 SMs x 32 per clk x 2.07 GHz; the kernel computes in 64-bit fixed "
+                               "point",
+                "multiply_adds_per_launch": mads, "flops_per_launch": flops,
+                "algorithmic_tflops": flops / (avg_ms / 1e3) / 1e12, "avg_launch_ms": avg_ms}
     else:
-        roof = {"bound": "alu", "achieved": None, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": None,
+        roof = {"bound": "alu", "achieved": None, "peak": INT_MAD_PEAK_T, "unit": "T multiply-add/s", "frac": None,
                 "traffic": None, "kernel": dom}
 
     cpu = None
