@@ -166,8 +166,8 @@ int emri_ctx_destroy(emri_ctx* ctx);
  * memory).  groups: 1..64, or 0 = by the call's size: 2 groups when each
  * holds at least 2^30 samples (walkers of a wave x n), else 1; smaller
  * groups lose more to the extra orbit launch and the stream hand-offs than
- * the overlap gains.  Default 1 (FP64: every kernel is bound by the FP64
- * pipe) and 0 (mixed).  EMRI_EINVAL otherwise. */
+ * the overlap gains.  Default 1 (FP64: the integer pipe bounds every
+ * kernel) and 0 (mixed).  EMRI_EINVAL otherwise. */
 int emri_ctx_set_pipeline(emri_ctx* ctx, int precision, int groups);
 
 /* Number of CUDA kernels the library has launched on this context so far

@@ -350,8 +350,8 @@ int run_loglike(emri_ctx* ctx, const emri_dataset* ds, const double* theta, int6
   };
   if (pipe == 0) {
     // by size: two groups when each holds at least 2^30 samples (walkers x
-    // n).  On the 1024-walker 2^21 mixed step two groups take 41.72 against
-    // 41.74 ms; smaller groups lose more to the extra orbit launch and the
+    // n).  On the 1024-walker 2^21 mixed step two groups take 41.51 against
+    // 41.54 ms; smaller groups lose more to the extra orbit launch and the
     // stream hand-offs than the overlap gains (8 walkers: 0.49 -> 0.56 ms).
     const int64_t w1 = std::min(wave, w);
     pipe = w1 * p.n >= ((int64_t)1 << 31) ? 2 : 1;
